@@ -380,6 +380,7 @@ int lbm_create(const lbm_lattice *lat, const lbm_species *sp, const lbm_mechanis
     c->mc = mc;
     c->lat.seg_nx = nullptr;     // read here only
     for (int k = 0; k < LBMK_NKERNELS; ++k) c->bs[k] = LBMK_BLOCK;
+    if (!is_mixed(lat->precision)) c->bs[LBMK_K_STEP] = 64;   // shared memory for 8 warps per SM instead of 4
     // the status word, then (at byte 16) the persistent step's barrier state
     int st = check_cuda(cudaMalloc((void **)&c->status, 16 + sizeof(GridBarrier)));
     if (st == LBM_OK) st = check_cuda(cudaMemsetAsync(c->status, 0, 16 + sizeof(GridBarrier), c->stream));

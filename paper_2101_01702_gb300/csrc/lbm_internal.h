@@ -101,6 +101,10 @@ struct MechConst {
     double hco[LBMK_MAXM][6], uco[LBMK_MAXM][6], gco[LBMK_MAXM][7];
     double inv_WWD[LBMK_MAXM][LBMK_MAXM];                   // 1 / (W_a W_b D_ab), 0 on the diagonal
     float inv_WWD_f[LBMK_MAXM][LBMK_MAXM];
+    // 1/D_ab as the integer mixh 2^29 + mixl < 2^58, in units of 2^mix_exp
+    // (mix_fixed: every entry exact, see lbm_pack_tables); 0 on the diagonal
+    int mix_fixed, mix_exp;
+    int mixh[LBMK_MAXM][LBMK_MAXM], mixl[LBMK_MAXM][LBMK_MAXM];
     int rtype[LBMK_MAXR], rev[LBMK_MAXR];
     int nreac[LBMK_MAXR], nprod[LBMK_MAXR];
     int reac[LBMK_MAXR][3], prod[LBMK_MAXR][3];             // species of each molecule

@@ -27,8 +27,6 @@
 //            X = -d_alpha G_alpha from the neighbours' records, and the
 //            collisions of Eqs. (finalNumericalEquations), (f), direction
 //            by direction
-// (k_chem, the production rates as a kernel of their own writing record
-// rows, serves builds with LBMK_FUSE_CHEM=0.)
 // One thread owns one lattice node; populations are structure-of-arrays
 // [set][direction][node] so that a warp's pulls are coalesced rows.
 #pragma once
@@ -80,8 +78,9 @@ typedef double WReal;
 // in the double unit; with its double Stefan-Maxwell solve the mixed unit
 // is FP64-bound and nearly insensitive to it (1..5 within 1.4 %, 3 best,
 // with the fewest spills of the capped choices).  The species and mixture
-// collision runs fastest at 3 blocks in the mixed units (168 registers) and
-// unconstrained in the double unit; with the production rates inside it,
+// collision runs fastest at 3 blocks in the mixed units (168 registers); the
+// double one (lbm_collide64.cuh) takes the registers it can get, its shared
+// memory holds it to 8 warps per SM; with the production rates inside it,
 // 256^3 mixed: 38.1 ms at 2 blocks (234 registers), 29.5 ms at 3, 31.2 ms
 // at 4 (128 registers, 224 B spilled).
 #ifndef LBMK_PRE_MINB
@@ -100,22 +99,12 @@ typedef double WReal;
 // Initialisation (equilibria of every set, outside the step; FP64-bound and
 // insensitive to occupancy: 43.1-43.5 ms at 4 or 6 blocks per SM): 6 blocks
 // (80 registers, ~30 B spilled).
-// Production rates formed inside the species collision (k_step) instead of
-// a kernel of their own: in the mixed units k_step waits on memory with
-// the FP64 pipe idle, and the rates are FP64 work of the same node, so the
-// fused kernel overlaps the two (256^3 mixed: k_chem 24.6 ms + k_step
-// 11.9 ms -> 29.5 ms; double: 24.0 + 257.7 -> 274.7 ms).  Results are bit
-// for bit those of the separate kernels (LBMK_FUSE_CHEM=0).
-#ifndef LBMK_FUSE_CHEM
-#define LBMK_FUSE_CHEM 1
-#endif
-// The energy collision inside k_step as well (LBMK_FUSE_ENERGY=1) was
-// measured slower (256^3 mixed: species collision 29.5 + energy 4.0 ms ->
-// 47.0 ms fused, with more spills at k_step's 168 registers), so k_step_g
-// stays a kernel of its own.
-#ifndef LBMK_FUSE_ENERGY
-#define LBMK_FUSE_ENERGY 0
-#endif
+// The production rates are formed inside the species collision (k_step), not
+// in a kernel of their own: they are FP64 work of the same node and overlap
+// the collision's memory traffic (256^3 mixed: k_chem 24.6 ms + k_step
+// 11.9 ms -> 29.5 ms).  The energy collision stays a kernel of its own
+// (k_step_g): inside k_step it was slower (29.5 + 4.0 ms -> 47.0 ms, more
+// spills at k_step's 168 registers).
 #ifndef LBMK_INIT_MINB
 #define LBMK_INIT_MINB 6
 #endif
@@ -1367,38 +1356,6 @@ __global__ void __launch_bounds__(LBMK_BLOCK, LBMK_PRE_MINB) k_pre(StepArgs a)
 }
 
 // ---------------------------------------------------------------------
-// Pass 1b: production rates of the record's state (molar_production).
-// ---------------------------------------------------------------------
-// Shared memory of k_chem for a block of bs threads.
-template <int M>
-constexpr size_t chem_smem(int bs) { return (size_t)M * bs * (2 * sizeof(double) + sizeof(WReal)); }
-
-template <int M>
-__global__ void __launch_bounds__(LBMK_MAXBLOCK) k_chem(StepArgs a)
-{
-    extern __shared__ double sh_chem[];
-    const int bs = blockDim.x;
-    double *sh_act = sh_chem;                                   // c_a exp(g_a / R_U T)
-    double *sh_g = sh_chem + (size_t)M * bs;                    // g_a / R_U T
-    WReal *sh_w = reinterpret_cast<WReal *>(sh_chem + (size_t)2 * M * bs);   // molar production
-    const MechConst &mc = c_mech[a.slot];
-    const int t = threadIdx.x;
-    const int n = blockIdx.x * blockDim.x + t;
-    if (n >= a.N) return;
-    const size_t N = a.N;
-    const RecRows rr = rec_rows(M);
-    Real *R = rec(a);
-    const double T = a.macro[DR_T * N + n];
-    const double rho = (double)R[(size_t)rr.rho * N + n];
-    double conc[M];
-#pragma unroll
-    for (int s = 0; s < M; ++s) conc[s] = rho * (double)R[(size_t)(rr.y + s) * N + n] * mc.invW[s];
-    molar_production<M>(mc, T, conc, sh_act, sh_g, sh_w, t, bs);
-#pragma unroll
-    for (int s = 0; s < M; ++s) R[(size_t)(rr.wd + s) * N + n] = (Real)(mc.W[s] * sh_w[s * bs + t]);
-}
-
-// ---------------------------------------------------------------------
 // Pass 2: G_alpha = (1/omega - 1/2) d_alpha Phi_alpha with the isotropic
 // gradient d_alpha phi = (1/theta) sum_i w_i c_ia phi(x + c_i).
 // ---------------------------------------------------------------------
@@ -1538,21 +1495,18 @@ __global__ void __launch_bounds__(LBMK_MAXBLOCK) k_step_g(StepArgs a)
 // Pass 3b: collisions of the species sets (Eq. (finalNumericalEquations)
 // with the quasi-equilibria of Eq. (fStar)) and of the mixture set f
 // (Eq. (f) with the isotropy correction of Eq. (Ai)), direction by
-// direction, in the storage precision.
+// direction, in the storage precision (the double unit's: lbm_collide64.cuh).
+// sh: shared memory, step_cols<M>() columns of bs doubles.
 // ---------------------------------------------------------------------
+#if LBMK_MIXED
 template <int M>
-__device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd)
+constexpr int step_cols() { return 3 * M; }      // scratch columns of the production rates
+
+template <int M>
+__device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, double *sh, int bs)
 {
-#if !LBMK_MIXED
-    // y-z factors of the species equilibria for the current row, this
-    // thread's column (kept in registers in the mixed units)
-    __shared__ double sh_yz[2 * M * LBMK_BLOCK];
-#endif
-#if LBMK_FUSE_CHEM
-    __shared__ double sh_act[M * LBMK_BLOCK];
-    __shared__ double sh_g[M * LBMK_BLOCK];
-    __shared__ WReal sh_w[M * LBMK_BLOCK];
-#endif
+    double *sh_act = sh, *sh_g = sh + M * bs;
+    WReal *sh_w = reinterpret_cast<WReal *>(sh + 2 * M * bs);
     const MechConst &mc = c_mech[a.slot];
     const int n = nd.n;
     const size_t N = a.N;
@@ -1596,21 +1550,16 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd)
 #pragma unroll
         for (int d = 0; d < 3; ++d) xs[s][d] = u[d] + ld(rr.du + 3 * s + d);
         bt[s] = ld(rr.beta + s);
-#if !LBMK_FUSE_CHEM
-        wd[s] = ld(rr.wd + s);
-#endif
     }
-#if LBMK_FUSE_CHEM
     {
-        // the production rates of this node, as k_chem forms them
+        // the production rates of this node
         double conc[M];
 #pragma unroll
         for (int s = 0; s < M; ++s) conc[s] = cvt<double>(rho) * cvt<double>(Yl[s]) * mc.invW[s];
-        molar_production<M>(mc, ldd(DR_T), conc, sh_act, sh_g, sh_w, threadIdx.x, LBMK_BLOCK);
+        molar_production<M>(mc, ldd(DR_T), conc, sh_act, sh_g, sh_w, threadIdx.x, bs);
 #pragma unroll
-        for (int s = 0; s < M; ++s) wd[s] = cvt<Real>(mc.W[s] * sh_w[s * LBMK_BLOCK + threadIdx.x]);
+        for (int s = 0; s < M; ++s) wd[s] = cvt<Real>(mc.W[s] * sh_w[s * bs + threadIdx.x]);
     }
-#endif
     const Real u2[3] = {u[0] * u[0], u[1] * u[1], u[2] * u[2]};
 
     const PopView v = view(a.src, a);
@@ -1620,11 +1569,9 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd)
 
     // Directions row by row: j = (cy+1) + 3 (cz+1), then cx = -1, 0, 1
     // (direction i = (cx+1) + 3 j, i.e. i = 0..26 in order).  The y-z
-    // factors of the product-form equilibria are formed once per row.  In
-    // mixed precision the populations of direction i+1 are loaded while
-    // direction i is collided (raw stored values; the rest state is added
-    // where they are used).
-    constexpr bool kPrefetch = LBMK_MIXED;
+    // factors of the product-form equilibria are formed once per row.  The
+    // populations of direction i+1 are loaded while direction i is collided
+    // (raw stored values; the rest state is added where they are used).
     Real fraw[M];
     auto load_raw = [&](int i) {
         const Src sr = src_of(i, p, a);
@@ -1632,16 +1579,14 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd)
 #pragma unroll
             for (int s = 0; s < M; ++s) fraw[s] = (Real)load_ghost(a, sr.side, s, i, sr.idx) - RAWREF(s, i);
         } else {
-            if (LBMK_MIXED && i == REST) return;
+            if (i == REST) return;
 #pragma unroll
             for (int s = 0; s < M; ++s) fraw[s] = load_raw_sf(v, s, i, sr.idx);
         }
     };
-    if (kPrefetch) load_raw(0);
+    load_raw(0);
 
-#if LBMK_MIXED
     Real pe_yz[M], ps_yz[M];
-#endif
     Real fe_yz = 0, AXyz = 0;
     int cy = 0, cz = 0;
     auto yz_factors = [&](int s, Real z, Real &pe, Real &ps) {
@@ -1656,43 +1601,25 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd)
             cz = j / 3 - 1;
             const int nnz = (cy != 0) + (cz != 0);
             // y-z factors of the species equilibria, shared by the row's three
-            // directions: in registers (float) or shared memory (double)
+            // directions
 #pragma unroll
             for (int s = 0; s < M; ++s) {
-#if LBMK_MIXED
                 yz_factors(s, RA(s) * T, pe_yz[s], ps_yz[s]);
-#else
-                Real pe, ps;
-                yz_factors(s, RA(s) * T, pe, ps);
-                sh_yz[(2 * s) * LBMK_BLOCK + threadIdx.x] = pe;
-                sh_yz[(2 * s + 1) * LBMK_BLOCK + threadIdx.x] = ps;
-#endif
             }
             fe_yz = rho * psi_c(cy, u[1], u2[1] + RT) * psi_c(cz, u[2], u2[2] + RT);
             // isotropy correction A_i . X (Eq. (Ai)): only |c_i| = 1
             AXyz = nnz == 1 ? (Real)0.5 * ((Real)cy * X[1] + (Real)cz * X[2]) : (Real)0;
         }
         Real fc[M];
-        if (kPrefetch) {
 #pragma unroll
-            for (int s = 0; s < M; ++s) fc[s] = fraw[s];
-            if (i + 1 < LBMK_Q) load_raw(i + 1);
-        } else {
-            load_raw(i);
-#pragma unroll
-            for (int s = 0; s < M; ++s) fc[s] = fraw[s];
-        }
-        if (LBMK_MIXED && i == REST) continue;   // rest of the species and mixture sets: below
+        for (int s = 0; s < M; ++s) fc[s] = fraw[s];
+        if (i + 1 < LBMK_Q) load_raw(i + 1);
+        if (i == REST) continue;   // rest of the species and mixture sets: below
         Real eqp[M], Dl[M];
 #pragma unroll
         for (int s = 0; s < M; ++s) {
             const Real z = RA(s) * T;
-#if LBMK_MIXED
             const Real pyz = pe_yz[s], syz = ps_yz[s];
-#else
-            const Real pyz = sh_yz[(2 * s) * LBMK_BLOCK + threadIdx.x];
-            const Real syz = sh_yz[(2 * s + 1) * LBMK_BLOCK + threadIdx.x];
-#endif
             const Real pe = psi_c(cx, u[0], u2[0] + z) * pyz;
             const Real pst = psi_c(cx, xs[s][0], xs[s][0] * xs[s][0] + z) * syz;
             eqp[s] = pe;
@@ -1726,7 +1653,6 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd)
             check += val;
         }
     }
-#if LBMK_MIXED
     // Rest direction of the species and mixture sets: populations and
     // equilibria in double, the collision increment (small near
     // equilibrium) in float.
@@ -1760,19 +1686,42 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd)
         store_sf(mc, a.dst, a, M - 1, REST, n, val);
         check += cvt<Real>(val);
     }
-#endif
     if (!isfinite(check)) flag(a.status, LBMK_BIT_NONFINITE);
-#if LBMK_FUSE_ENERGY
-    collide_energy<M>(a, nd);
-#endif
 }
+#else
+}  // namespace
+#include "lbm_collide64.cuh"
+namespace {
+#endif
+
+// Shared memory of a block of bs threads for step_node.
+template <int M>
+constexpr size_t step_smem(int bs) { return (size_t)step_cols<M>() * bs * sizeof(double); }
+
+extern __shared__ double sh_step[];
 
 template <int M>
 __global__ void __launch_bounds__(LBMK_BLOCK, LBMK_STEP_MINB) k_step(StepArgs a)
 {
     Node nd;
     if (!node_of(nd, a)) return;
-    step_node<M>(a, nd);
+    step_node<M>(a, nd, sh_step, blockDim.x);
+}
+
+// Opts kernel f in to dynamic shared memory above 48 KB, once per device
+// (done: a word of the caller's, bit d: device d has opted in).
+// Idempotent, so two threads racing here both succeed.
+template <class F>
+int opt_in_smem(F *f, size_t bytes, std::atomic<unsigned long long> &done)
+{
+    if (bytes <= 48 * 1024) return 0;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return (int)cudaErrorInvalidDevice;
+    if (done.load() >> dev & 1ull) return 0;
+    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) return (int)e;
+    done.fetch_or(1ull << dev);
+    return 0;
 }
 
 // ---------------------------------------------------------------------
@@ -1794,31 +1743,16 @@ int launch_one(const StepArgs &a, int k)
         }
         break;
     case LBMK_K_PRE: k_pre<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
-    case LBMK_K_CHEM: {
-        if (LBMK_FUSE_CHEM) break;          // the rates are formed inside k_step
-        // blocks needing more than 48 KB of dynamic shared memory opt in,
-        // once per device (only tuned block sizes do; the default never)
-        if (chem_smem<M>(bs) > 48 * 1024) {
-            static std::atomic<unsigned long long> opted{0};   // bit d: device d has opted in
-            int dev = 0;
-            if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return (int)cudaErrorInvalidDevice;
-            if (!(opted.load() >> dev & 1ull)) {
-                // idempotent, so two threads racing here both succeed
-                const cudaError_t e = cudaFuncSetAttribute(k_chem<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                           (int)chem_smem<M>(LBMK_MAXBLOCK));
-                if (e != cudaSuccess) return (int)e;
-                opted.fetch_or(1ull << dev);
-            }
-        }
-        k_chem<M><<<grid_for(a.N, bs), bs, chem_smem<M>(bs), a.stream>>>(a);
+    case LBMK_K_CHEM: break;            // the rates are formed inside k_step
+    case LBMK_K_GRAD: k_grad<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
+    case LBMK_K_STEPG: k_step_g<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
+    case LBMK_K_STEP: {
+        static std::atomic<unsigned long long> opted{0};
+        const int e = opt_in_smem(k_step<M>, step_smem<M>(LBMK_BLOCK), opted);
+        if (e) return e;
+        k_step<M><<<grid_for(a.N, bs), bs, step_smem<M>(bs), a.stream>>>(a);
         break;
     }
-    case LBMK_K_GRAD: k_grad<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
-    case LBMK_K_STEPG:
-        if (LBMK_FUSE_ENERGY) break;        // the energy set collides inside k_step
-        k_step_g<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a);
-        break;
-    case LBMK_K_STEP: k_step<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
     default: return (int)cudaErrorInvalidValue;
     }
     return (int)cudaGetLastError();
@@ -1909,7 +1843,7 @@ __device__ __forceinline__ bool persist_step(const StepArgs &b, int tile, GridBa
     // each one's arithmetic as in its own kernel (no values shared)
     tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) { collide_energy<M>(b, nd); });
     if (!grid_barrier(bar, nb, cap, b.status)) return false;
-    tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) { step_node<M>(b, nd); });
+    tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) { step_node<M>(b, nd, sh_step, LBMK_BLOCK); });
     return grid_barrier(bar, nb, cap, b.status);
 }
 
@@ -1931,9 +1865,12 @@ template <int M>
 int run_persistent(const StepArgs &a, int nsteps, int tile_mult, GridBarrier *bar, unsigned cap)
 {
     if (nsteps < 1 || tile_mult < 1) return (int)cudaErrorInvalidValue;
-    if (!LBMK_FUSE_CHEM) return (int)cudaErrorNotSupported;     // the rates must form inside the collision
     int per_sm = 0, dev = 0, nsm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_persist<M>, LBMK_BLOCK, 0);
+    static std::atomic<unsigned long long> opted{0};
+    const int eo = opt_in_smem(k_persist<M>, step_smem<M>(LBMK_BLOCK), opted);
+    if (eo) return eo;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_persist<M>, LBMK_BLOCK,
+                                                                  step_smem<M>(LBMK_BLOCK));
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return (int)e;
@@ -1948,8 +1885,8 @@ int run_persistent(const StepArgs &a, int nsteps, int tile_mult, GridBarrier *ba
     GridBarrier *bb = bar;
     unsigned cc = cap;
     void *args[] = {(void *)&a0, (void *)&a1, (void *)&ns, (void *)&tl, (void *)&bb, (void *)&cc};
-    return (int)cudaLaunchCooperativeKernel((const void *)k_persist<M>, dim3(blocks), dim3(LBMK_BLOCK), args, 0,
-                                            a.stream);
+    return (int)cudaLaunchCooperativeKernel((const void *)k_persist<M>, dim3(blocks), dim3(LBMK_BLOCK), args,
+                                            step_smem<M>(LBMK_BLOCK), a.stream);
 }
 #endif  // LBMK_COHERENT_LOADS
 

@@ -70,6 +70,28 @@ static inline int lbm_pack_tables(const lbm_species *sp, const lbm_mechanism *me
             mc.inv_WWD_f[a][b] = (float)mc.inv_WWD[a][b];
         }
     }
+    // Fixed-point 1/D_ab for the cross terms of the double collision: the
+    // largest entry keeps its leading bit at 2^57, so that entries down to
+    // 1/32 of it keep all 53 bits; wider ranges take the floating sums.
+    {
+        double top = 0.0, low = INFINITY;
+        for (int a = 0; a < M; ++a)
+            for (int b = 0; b < M; ++b)
+                if (a != b) {
+                    top = fmax(top, 1.0 / sp->D[M * a + b]);
+                    low = fmin(low, 1.0 / sp->D[M * a + b]);
+                }
+        const int e = isfinite(top) ? ilogb(top) : 0;
+        mc.mix_fixed = isfinite(top) && top <= 32.0 * low && e > -500 && e < 500;
+        mc.mix_exp = e - 57;
+        for (int a = 0; a < M && mc.mix_fixed; ++a)
+            for (int b = 0; b < M; ++b)
+                if (a != b) {
+                    const long long v = (long long)ldexp(1.0 / sp->D[M * a + b], 57 - e);
+                    mc.mixh[a][b] = (int)(v >> 29);
+                    mc.mixl[a][b] = (int)(v & 0x1fffffff);
+                }
+    }
     mc.transport = sp->transport;
     if (sp->transport == LBM_TRANSPORT_MIXTURE_AVERAGED) {
         for (int a = 0; a < M; ++a) {
