@@ -101,6 +101,7 @@ extern "C" int lbm_step_fixed_scratch(const lbm_lattice *lat, const lbm_species 
     a.nz = lat->nz;
     a.N = (int)N;
     a.bc_x = lat->bc_x;
+    a.fixed = mc.mix_fixed;
     a.nseg = 0;
     a.xseg = nullptr;
     a.segs = nullptr;

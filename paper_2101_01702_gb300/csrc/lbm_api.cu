@@ -188,6 +188,7 @@ StepArgs args_of(const lbm_ctx *c)
     a.nz = c->lat.nz;
     a.N = c->N;
     a.bc_x = c->lat.bc_x;
+    a.fixed = c->mc.mix_fixed;
     for (int k = 0; k < LBMK_NKERNELS; ++k) a.bs[k] = c->bs[k];
     a.nseg = c->nseg;
     a.xseg = c->xseg;

@@ -43,7 +43,7 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
     const MechConst &mc = c_mech[a.slot];
     const int n = nd.n, t = threadIdx.x;
     const size_t N = a.N;
-    const RecRows rr = rec_rows(M);
+    const RecRows rr = rec_rows(M, LBMK_MIXED);
     const double *R = rec(a);
     auto ld = [&](int row) { return R[(size_t)row * N + n]; };
 

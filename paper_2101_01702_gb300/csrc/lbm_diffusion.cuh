@@ -1,0 +1,270 @@
+// Stefan-Maxwell diffusion velocities (Eq. (transform1)) without the FP64
+// pipe: a float factorisation and one step of iterative refinement whose
+// residual is formed in fixed point (lbm_fixed.cuh).  For the mixed unit,
+// where the velocities are stored as floats.
+//
+// The system of a node, with h = kappa/2 = m R_U T/2, A_ab = 1/(W_a W_b D_ab),
+//   x_a + h sum_b A_ab Y_b (x_a - x_b) = V_a,   V_a = j_a/rho_a - u,
+// is diagonally dominant by rows with excess 1, and A is symmetric.
+// Eliminating species k leaves a system of the same form with
+//   A_ij += A_ik A_kj Y_k / d_k,   e_i += A_ik Y_k e_k / d_k,
+//   d_k = e_k + sum_{j>k} A_kj Y_j            (e = 1/h at the start),
+// sums of positive terms only (Grassmann, Taksar and Heyman's elimination),
+// so the float factors carry a few units of 2^-24 in every entry, however
+// small the mass fractions.  The float solution x0, rounded to integers below
+// 2^29, is an exact operand of the residual
+//   r_a = V_a - x_a - (h/W_a) (x_a S_a - sum_b K_ab n_b x_b),
+//   S_a = sum_b K_ab n_b,  K_ab = 1/D_ab,  n_b = Y_b/W_b,
+// whose sums over b run in 58-bit limbs (S_a and the last differences in
+// pairs of floats), 2^-45 of their largest term; the correction, solved with the same
+// factors, is then good to 2^-40 of x, and x0 plus it is rounded to float
+// once -- the float that the double solution rounds to, but for ties
+// (tests/test_gpu_diffusion.py measures both against 64-bit solutions).
+//
+// A double LDL^T solve costs 740 FP64 instructions per warp at nine species,
+// 56 thousand cycles of a scheduler; this one about 7 thousand
+// integer and float instructions.
+#pragma once
+
+#include "lbm_fixed.cuh"
+
+namespace {
+
+// a + b as a rounded sum and its error (Knuth).
+__device__ __forceinline__ float two_sum(float a, float b, float &err)
+{
+    const float s = a + b, bb = s - a;
+    err = (a - (s - bb)) + (b - bb);
+    return s;
+}
+
+// The leading 24 and the next 23 bits of d as floats (0 below the float
+// range; d within it above).
+__device__ __forceinline__ void split2(double d, float &h, float &l)
+{
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const int ed = (int)((hi >> 20) & 0x7ffu) - 896;                 // float exponent field
+    const unsigned sign = hi & 0x80000000u;
+    const unsigned man = ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const bool ok = ed > 24;
+    h = ok ? __uint_as_float(sign | ((unsigned)ed << 23) | man) : 0.0f;
+    // 23 of the low 29 bits as a float of exponent ed - 23, less its implicit one
+    const unsigned e2 = sign | ((unsigned)(ed - 23) << 23);
+    l = ok ? __uint_as_float(e2 | ((lo & 0x1fffffffu) >> 6)) - __uint_as_float(e2) : 0.0f;
+}
+
+// 2^k, clamped to the normal floats.
+__device__ __forceinline__ float pow2f(int k)
+{
+    return __int_as_float((min(max(k, -126), 127) + 127) << 23);
+}
+
+__device__ __forceinline__ float rcp_approx(float x)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return 1.0f / x;
+#endif
+}
+
+// du[M][3], and ita = 1/tau_a [M], of a node, from the rows (stride N) of
+// its species densities ra, velocity ud and momenta J, and hk = h/rho.  All
+// quantities are scale-free in the densities: with rho_b in place of Y_b, h
+// becomes h/rho.  sh: 2 M columns of this thread's shared memory, stride
+// bs.  Sets *bad for a non-finite pivot.
+template <int M>
+__device__ __forceinline__ void diffusion_refined(const MechConst &mc, const double *ra, const double *ud,
+                                                  const float *J, size_t N, double hk, double *sh, int bs,
+                                                  float (*du)[3], float *ita, bool *bad)
+{
+    // n_b = rho_b / W_b as limbs
+    int en = 0;
+    long long *ln = reinterpret_cast<long long *>(sh), *lS = ln + M * bs;
+    float y[M], nh[M], nl[M];
+    unsigned major = 0;                                    // species above 2^-16 of the largest n
+    {
+        double nb[M];
+#pragma unroll
+        for (int b = 0; b < M; ++b) {
+            const double r = ra[(size_t)b * N];
+            nb[b] = r * mc.invW[b];
+            en = max(en, biased_exponent(nb[b]));
+            float lo;
+            split2(r, y[b], lo);
+            y[b] += lo;
+        }
+#pragma unroll
+        for (int b = 0; b < M; ++b) {
+            split2(nb[b], nh[b], nl[b]);
+            const Limbs58 x = to_limbs58(nb[b], en);
+            ln[b * bs] = ((long long)x.h << 32) | (unsigned)x.l;
+            if (biased_exponent(nb[b]) + 16 >= en) major |= 1u << b;
+        }
+    }
+    float hh, hl;
+    split2(hk, hh, hl);
+    const int cs = mc.mix_exp + en - 1080 + 58;            // sums of K n are integers times 2^cs
+
+    // S_a as pairs of floats, summed with their errors (all terms have one
+    // sign, so each S_a keeps its relative accuracy), and 1/tau_a = 2 (h/W_a) S_a
+#pragma unroll
+    for (int s = 0; s < M; ++s) {
+        float Sh = 0.0f, Sl = 0.0f;
+#pragma unroll
+        for (int b = 0; b < M; ++b)
+            if (b != s) {
+                const float kh = mc.invD_h[s][b], p = kh * nh[b];
+                const float pe = fma(kh, nh[b], -p) + fma(kh, nl[b], mc.invD_l[s][b] * nh[b]);
+                float e;
+                Sh = two_sum(Sh, p, e);
+                Sl += e + pe;
+            }
+        const float S = Sh + Sl;
+        Sl = (Sh - S) + Sl;
+        lS[s * bs] = ((long long)__float_as_int(S) << 32) | (unsigned)__float_as_int(Sl);
+        const float wh = mc.invW_h[s], wl = mc.invW_l[s];
+        const float th = hh * wh, tl = fma(hh, wh, -th) + fma(hh, wl, hl * wh);
+        const float p = th * S;
+        ita[s] = 2.0f * (p + (fma(th, S, -p) + fma(th, Sl, tl * S)));
+    }
+
+    // factors: K[i][j], i < j, and 1/d_k
+    float K[M][M], dinv[M];
+    const float ex0 = rcp_approx(hh);
+    {
+        float ex[M];
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            ex[i] = ex0;
+#pragma unroll
+            for (int j = i + 1; j < M; ++j) K[i][j] = mc.inv_WWD_f[i][j];
+        }
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            float d = ex[k];
+#pragma unroll
+            for (int j = k + 1; j < M; ++j) d = fma(K[k][j], y[j], d);
+            if (!finite_bits(d)) *bad = true;
+            dinv[k] = rcp_approx(d);
+            const float m = y[k] * dinv[k];
+#pragma unroll
+            for (int i = k + 1; i < M; ++i) {
+                const float l = K[k][i] * m;
+                ex[i] = fma(l, ex[k], ex[i]);
+#pragma unroll
+                for (int j = i + 1; j < M; ++j) K[i][j] = fma(l, K[k][j], K[i][j]);
+            }
+        }
+    }
+    // x <- solution for the right-hand side x (in units of V)
+    auto solve = [&](float *x) {
+#pragma unroll
+        for (int k = 0; k < M; ++k) x[k] *= ex0;
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            const float mk = y[k] * dinv[k] * x[k];
+#pragma unroll
+            for (int i = k + 1; i < M; ++i) x[i] = fma(K[k][i], mk, x[i]);
+        }
+        float z[M];
+#pragma unroll
+        for (int k = M - 1; k >= 0; --k) {
+            float s = x[k];
+#pragma unroll
+            for (int j = k + 1; j < M; ++j) s = fma(K[k][j], z[j], s);
+            x[k] = s * dinv[k];
+            z[k] = y[k] * x[k];
+        }
+    };
+
+#pragma unroll 1
+    for (int d = 0; d < 3; ++d) {
+        // V_a = j_a / rho_a - u as pairs of floats; 0 for an absent species
+        float Vh[M], Vl[M], x[M];
+        float uh, ul;
+        split2(ud[d * N], uh, ul);
+#pragma unroll
+        for (int s = 0; s < M; ++s) {
+            float rh, rl;
+            split2(ra[(size_t)s * N], rh, rl);
+            const float j = J[(size_t)(3 * s + d) * N];
+            const float ri = rcp_approx(rh), q = j * ri;
+            const float q1 = fma(-q, rl, fma(-q, rh, j)) * ri;
+            float e;
+            const float s1 = two_sum(q, -uh, e);
+            const bool here = rh != 0.0f;
+            Vh[s] = here ? s1 : 0.0f;
+            Vl[s] = here ? e + (q1 - ul) : 0.0f;
+            x[s] = Vh[s] + Vl[s];
+        }
+        solve(x);
+        // x0 as integers below 2^29 times 2^-kx, the scale set by the largest
+        // x of a major species; a minor species beyond it by a factor 2^f
+        // takes 2^(f-kx), and starts from zero if its n x0 is beyond the
+        // scale of the sums
+        int em = 0;
+#pragma unroll
+        for (int s = 0; s < M; ++s)
+            if (major >> s & 1u) em = max(em, (__float_as_int(x[s]) >> 23) & 0xff);
+        const int e0 = min(max(em, 65), 200), kx = 155 - e0;                  // |x0| < 2^(e0 - 126)
+        const int c = cs + 30 - kx;                                           // the sums are integers times 2^c
+        const float g1 = pow2f(41 + c), g2 = pow2f(18 + c), g3 = c < -126 ? 0.0f : pow2f(c);
+        Limbs58 w[M];
+#pragma unroll
+        for (int s = 0; s < M; ++s) {
+            const int e = (__float_as_int(x[s]) >> 23) & 0xff, f = min(max(e - e0, 0), 41);
+            int xi = __float2int_rn(x[s] * pow2f(kx - f));
+            const long long v = ln[s * bs];
+            long long ph = (long long)(int)(v >> 32) * xi, pl = (long long)(int)v * xi;
+            if (f > 0 && (f > 40 || ((ph < 0 ? -ph : ph) >> (58 - f)) != 0)) {
+                xi = 0;
+                ph = pl = 0;
+            }
+            const long long p = f == 0 ? (ph >> 1) + (pl >> 30)
+                                       : (ph << (f - 1)) + (f <= 30 ? pl >> (30 - f) : pl << (f - 30));
+            w[s] = Limbs58{(int)(p >> 29), (int)((unsigned)p & 0x1fffffffu)};
+            x[s] = (float)xi * pow2f(f - kx);
+        }
+        float r[M];
+#pragma unroll
+        for (int s = 0; s < M; ++s) {
+            long long hi = 0, mid = 0;
+#pragma unroll
+            for (int b = 0; b < M; ++b)
+                if (b != s) fma_limbs58(hi, mid, mc.mixh[s][b], mc.mixl[s][b], w[b]);
+            const long long G = hi + (mid >> 29);
+            // G as a pair of floats, from pieces of 22, 23 and 18 bits
+            const float G1 = (__int_as_float(0x4b400000 + (int)(G >> 41)) - 12582912.0f) * g1;
+            const float G2 = (__int_as_float(0x4b000000 | (int)((G >> 18) & 0x7fffff)) - 8388608.0f) * g2;
+            const float G3 = (__int_as_float(0x4b000000 | (int)(G & 0x3ffff)) - 8388608.0f) * g3;
+            const float Gh = G1 + G2, Gl = (G2 - (Gh - G1)) + G3;
+            const long long S = lS[s * bs];
+            const float x0 = x[s];
+            // H = x_a S_a - G_a
+            const float Sh = __int_as_float((int)(S >> 32)), xS = x0 * Sh;
+            float He;
+            const float Hh = two_sum(xS, -Gh, He);
+            const float Hl = He + (fma(x0, Sh, -xS) + fma(x0, __int_as_float((int)S), -Gl));
+            const float wh = mc.invW_h[s], wl = mc.invW_l[s];
+            const float th = hh * wh, tl = fma(hh, wh, -th) + fma(hh, wl, hl * wh);
+            const float p = th * Hh, pe = fma(th, Hh, -p) + fma(th, Hl, tl * Hh);
+            float e1, e2;
+            const float s1 = two_sum(Vh[s], -x0, e1);
+            const float s2 = two_sum(s1, -p, e2);
+            r[s] = s2 + (e2 + ((e1 + Vl[s]) - pe));
+        }
+        solve(r);
+#pragma unroll
+        for (int s = 0; s < M; ++s) {
+            const float v = Vh[s] == 0.0f && Vl[s] == 0.0f && y[s] == 0.0f ? 0.0f : x[s] + r[s];
+            if (d == 0) du[s][0] = v;
+            else if (d == 1) du[s][1] = v;
+            else du[s][2] = v;
+        }
+    }
+}
+
+}  // namespace

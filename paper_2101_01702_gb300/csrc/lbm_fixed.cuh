@@ -3,11 +3,11 @@
 //
 // Measured on GB300 (one SM, 32 warps): a double multiply-add takes 19
 // cycles per warp instruction, a 32 x 32 + 64 bit integer multiply-add 1.3.
-// Three of the latter give a product of two 58-bit numbers to 2^-58, so a
+// Three of the latter give a product of two 58-bit numbers to 2^-56, so a
 // sum of products over operands brought to a common exponent is formed at
-// about a fifth of the FP64 pipe's cost, and with less error than
-// a chain of fused multiply-adds: the operands keep all 53 bits down to
-// 2^-5 of the largest one, and the sum is rounded once.
+// about a fifth of the FP64 pipe's cost, with no more error than a chain
+// of fused multiply-adds: the operands keep all 53 bits down to 2^-5 of the
+// largest one, and the sum is rounded once.
 #pragma once
 
 #include "lbm_internal.h"
@@ -36,8 +36,8 @@ __device__ __forceinline__ Limbs58 to_limbs58(double d, int e)
 }
 
 // Adds x (limbs) times the constant (ch, cl) < 2^58 to a running sum kept
-// as hi + mid 2^-29 in units of 2^58; the low x low product, below
-// 2^-58 of the largest term, is left out.  Eight terms stay within 63 bits.
+// as hi + mid 2^-29 in units of 2^58; the low x low product, less than
+// one of those units, is left out.  Eight terms stay within 63 bits.
 __device__ __forceinline__ void fma_limbs58(long long &hi, long long &mid, int ch, int cl, Limbs58 x)
 {
     hi += (long long)ch * x.h;

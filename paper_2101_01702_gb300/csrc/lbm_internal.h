@@ -8,6 +8,7 @@
 
 #define LBMK_MAXM 12
 #define LBMK_MAXS (LBMK_MAXM + 1)
+#define LBMK_MIXM 9
 #define LBMK_MAXR 32
 #define LBMK_SLOTS 4
 #define LBMK_Q 27
@@ -35,12 +36,16 @@ struct GridBarrier {
 //   DR_FEQ0   rest-direction equilibrium of the species and mixture sets (M)
 //   DR_GE     rho E            DR_GQ  q^eq (3)       DR_GR  R^eq - rho E theta I (6: xx yy zz xy xz yz)
 //   DR_GTR    tr(R^eq - rho E theta I) / 3
+//   in mixed precision also DR_RA rho_a (M), DR_U u (3), DR_HK kappa/(2 rho)
+//   (fast mixed: 1/rho): what the diffusion pass (k_diff) needs in double
 // Storage-type rows:
 //   nup  1/omega - 1/2      phi  Phi (3)        g    G (3)
 //   y    Y_a (M)            rho  rho            u    u (3)
-//   du   du_a (3M, a-major) wd   rho_dot_a (M; written only by k_chem)  beta beta_a (M)
+//   du   du_a (3M, a-major; until k_diff the momenta j_a)   beta beta_a (M)
+//   ra   rho_a (M; double precision only)
 //   kappa m R_U T           rt   R T            om   omega      om1 omega_1
-//   p    P                  dq   (omega - omega_1)(q* - q^eq) without the grad-Y part (3)
+//   p    P                  dq   (omega - omega_1)(q* - q^eq) without the grad-Y part (3; until k_diff
+//                                also without the part of the diffusion velocities)
 //   h    H_a (M)
 #define DR_T 0
 #define DR_FEQ0 1
@@ -48,19 +53,23 @@ __host__ __device__ constexpr int dr_ge(int M) { return M + 1; }
 __host__ __device__ constexpr int dr_gq(int M) { return M + 2; }
 __host__ __device__ constexpr int dr_gr(int M) { return M + 5; }
 __host__ __device__ constexpr int dr_gtr(int M) { return M + 11; }
-__host__ __device__ constexpr int macro_double_rows(int M) { return M + 12; }
+__host__ __device__ constexpr int dr_ra(int M) { return M + 12; }
+__host__ __device__ constexpr int dr_u(int M) { return 2 * M + 12; }
+__host__ __device__ constexpr int dr_hk(int M) { return 2 * M + 15; }
+__host__ __device__ constexpr int macro_double_rows(int M, bool mixed) { return mixed ? 2 * M + 16 : M + 12; }
 struct RecRows {
-    int nup, phi, g, y, rho, u, du, wd, beta, kappa, rt, om, om1, p, dq, h, total;
+    int nup, phi, g, y, rho, u, du, beta, kappa, rt, om, om1, p, dq, h, ra, total;
 };
-__host__ __device__ constexpr RecRows rec_rows(int M)
+__host__ __device__ constexpr RecRows rec_rows(int M, bool mixed)
 {
-    return RecRows{0, 1, 4, 7, 7 + M, 8 + M, 11 + M, 11 + 4 * M, 11 + 5 * M, 11 + 6 * M, 12 + 6 * M, 13 + 6 * M,
-                   14 + 6 * M, 15 + 6 * M, 16 + 6 * M, 19 + 6 * M, 19 + 7 * M};
+    return RecRows{0, 1, 4, 7, 7 + M, 8 + M, 11 + M, 11 + 4 * M, 11 + 5 * M, 12 + 5 * M, 13 + 5 * M,
+                   14 + 5 * M, 15 + 5 * M, 16 + 5 * M, 19 + 5 * M, 19 + 6 * M, 19 + (mixed ? 6 : 7) * M};
 }
 // Bytes of the macro buffer for N nodes, M species and a storage element size.
 __host__ __device__ constexpr size_t macro_bytes_for(int M, size_t N, size_t real_size)
 {
-    return (size_t)macro_double_rows(M) * N * sizeof(double) + (size_t)rec_rows(M).total * N * real_size;
+    const bool mixed = real_size == sizeof(float);
+    return (size_t)macro_double_rows(M, mixed) * N * sizeof(double) + (size_t)rec_rows(M, mixed).total * N * real_size;
 }
 
 // Population buffer.
@@ -102,9 +111,13 @@ struct MechConst {
     double inv_WWD[LBMK_MAXM][LBMK_MAXM];                   // 1 / (W_a W_b D_ab), 0 on the diagonal
     float inv_WWD_f[LBMK_MAXM][LBMK_MAXM];
     // 1/D_ab as the integer mixh 2^29 + mixl < 2^58, in units of 2^mix_exp
-    // (mix_fixed: every entry exact, see lbm_pack_tables); 0 on the diagonal
+    // (mix_fixed: every entry exact, see lbm_pack_tables; at most LBMK_MIXM
+    // species, so that four slots fit constant memory); 0 on the diagonal;
+    // 1/W_a and 1/D_ab as pairs of floats
     int mix_fixed, mix_exp;
-    int mixh[LBMK_MAXM][LBMK_MAXM], mixl[LBMK_MAXM][LBMK_MAXM];
+    float invW_h[LBMK_MAXM], invW_l[LBMK_MAXM];
+    float invD_h[LBMK_MIXM][LBMK_MIXM], invD_l[LBMK_MIXM][LBMK_MIXM];
+    int mixh[LBMK_MIXM][LBMK_MIXM], mixl[LBMK_MIXM][LBMK_MIXM];
     int rtype[LBMK_MAXR], rev[LBMK_MAXR];
     int nreac[LBMK_MAXR], nprod[LBMK_MAXR];
     int reac[LBMK_MAXR][3], prod[LBMK_MAXR][3];             // species of each molecule
@@ -156,6 +169,7 @@ enum { LBMK_K_GHOST = 0, LBMK_K_PRE, LBMK_K_CHEM, LBMK_K_GRAD, LBMK_K_STEPG, LBM
 
 struct StepArgs {
     int slot, M, nx, ny, nz, N, bc_x;
+    int fixed;               // the tables' mix_fixed: kernels with fixed-point sums over the species
     int bs[LBMK_NKERNELS];   // threads per block of each kernel
     // Lattices side by side in x (nseg >= 2): per x coordinate its lattice's
     // x range and index {x0, x1, k, 0}; per lattice its range {x0, x1}.

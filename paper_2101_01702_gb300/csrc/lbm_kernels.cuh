@@ -38,6 +38,7 @@
 #include <type_traits>
 
 #include "lbm_internal.h"
+#include "lbm_fixed.cuh"
 
 #ifndef LBMK_FAST
 #define LBMK_FAST 0
@@ -71,20 +72,21 @@ typedef double WReal;
 #define INVWWD_S(a_, b_) (mc.inv_WWD[a_][b_])
 #endif
 
-// Minimum resident blocks per SM asked of the compiler for the two large
-// kernels (register budget 65536 / (LBMK_BLOCK * minB)).  Measured on the
-// 256^3 nine-species lattice: the moment pass runs fastest at 5 blocks in
-// the fast mixed unit (96 registers, some spilled; latency bound) and at 3
-// in the double unit; with its double Stefan-Maxwell solve the mixed unit
-// is FP64-bound and nearly insensitive to it (1..5 within 1.4 %, 3 best,
-// with the fewest spills of the capped choices).  The species and mixture
+// Minimum resident blocks per SM asked of the compiler for the large
+// kernels (register budget 65536 / (LBMK_BLOCK * minB)).  Measured, nine
+// species: the moment pass with the diffusion pass, 256^3 mixed, at 3 + 3
+// blocks 33.8 ms, 4 + 3 33.3, 3 + 4 32.2, 5 + 2 30.0 (6 + 2 and 5 + 1 the
+// same); 160^3 fast mixed 5.62 ms at 5 + 3, 5.43 at 5 + 5, 5.88 at 6 + 2;
+// 128^3 double 6.71 ms at 5 + 2, 6.75 at 4 + 4, 7.21 at 2 + 3.  The species and mixture
 // collision runs fastest at 3 blocks in the mixed units (168 registers); the
 // double one (lbm_collide64.cuh) takes the registers it can get, its shared
 // memory holds it to 8 warps per SM; with the production rates inside it,
-// 256^3 mixed: 38.1 ms at 2 blocks (234 registers), 29.5 ms at 3, 31.2 ms
-// at 4 (128 registers, 224 B spilled).
+// 256^3 mixed: 33.4 ms at 2 blocks, 27.6 ms at 3, 33.1 ms at 4.
 #ifndef LBMK_PRE_MINB
-#define LBMK_PRE_MINB (LBMK_MIXED && LBMK_FAST ? 5 : 3)
+#define LBMK_PRE_MINB 5
+#endif
+#ifndef LBMK_DIFF_MINB
+#define LBMK_DIFF_MINB (LBMK_FAST ? 5 : 2)
 #endif
 #ifndef LBMK_STEP_MINB
 #define LBMK_STEP_MINB (LBMK_MIXED ? 3 : 1)
@@ -428,7 +430,7 @@ __device__ __forceinline__ size_t nb_of(const StencilIdx &t, const StepArgs &a)
 
 __device__ __forceinline__ Real *rec(const StepArgs &a)
 {
-    return reinterpret_cast<Real *>(a.macro + (size_t)macro_double_rows(a.M) * a.N);
+    return reinterpret_cast<Real *>(a.macro + (size_t)macro_double_rows(a.M, LBMK_MIXED) * a.N);
 }
 
 // ---------------------------------------------------------------------
@@ -1130,67 +1132,164 @@ __global__ void __launch_bounds__(LBMK_BLOCK, LBMK_MOM_MINB) k_moments(StepArgs 
     }
 }
 
+#if LBMK_MIXED && !LBMK_FAST
+}  // namespace
+#include "lbm_diffusion.cuh"
+namespace {
+#endif
+
 // ---------------------------------------------------------------------
-// Pass 1: pull, moments, temperature, relaxation, Stefan-Maxwell solve;
-// writes the per-node record (all rows but the production rates).
+// Pass 1: pull, moments, temperature, relaxation, energy equilibrium
+// moments; writes the per-node record but for the diffusion velocities
+// (momenta j_a in their place), beta_a and the part of Dq that needs them.
+//
+// The loops over the species are not unrolled: fully unrolled, this pass
+// and the solve of pass 1b were 19,500 instructions run once per
+// warp, more than the instruction caches hold, and a quarter of every
+// warp's time went to fetching them.
+// sh: this thread's shared memory, pre_cols<M>() columns of bs doubles
+// (rho_a, then Y_a).
 // ---------------------------------------------------------------------
 template <int M>
-__device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd)
+constexpr int pre_cols() { return 2 * M; }
+
+template <int M>
+__device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd, double *sh, int bs)
 {
     const MechConst &mc = c_mech[a.slot];
-    PullIdx p;
-    make_pull(p, nd, a);
-    double rho_a[M];
-    Real ja[M][3];
-    Sums sm;
-    pull_moments<M, true>(mc, a, p, nd.n, rho_a, ja, sm);
-
-    // composition and velocity (Eq. (strongest) for the slaved species)
-    const double rho = sm.rho, ir = 1.0 / rho;
-    double rest = 0.0;
-#pragma unroll
-    for (int s = 0; s < M - 1; ++s) rest += rho_a[s];
-    rho_a[M - 1] = rho - rest;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        Real js = sm.jr[d];
-#pragma unroll
-        for (int s = 0; s < M - 1; ++s) js -= ja[s][d];
-        ja[M - 1][d] = js;
-    }
-    double Y[M], inv_m = 0.0;
-    bool neg = false;
-#pragma unroll
-    for (int s = 0; s < M; ++s) {
-        Y[s] = rho_a[s] * ir;
-        inv_m = fma(Y[s], mc.invW[s], inv_m);
-        if (__double2hiint(rho_a[s]) < 0)     // sign bit first: the compare only for negative values
-            neg |= rho_a[s] < -1e-10 * rho;  // below rounding noise of trace species
-    }
-    if (!(rho > 0.0) || !isfinite(sm.rhoE)) flag(a.status, LBMK_BIT_NONFINITE);
-    if (neg) flag(a.status, LBMK_BIT_NEGATIVE);
-    const double u[3] = {sm.j[0] * ir, sm.j[1] * ir, sm.j[2] * ir};
-    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-
-    // temperature, Eq. (temperature)
     const int n = nd.n;
     const size_t N = a.N;
-    double T, Cv = 0.0;
+    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    Real *R = rec(a);
+    const PopView v = view(a.src, a);
+    PullIdx p;
+    make_pull(p, nd, a);
+    // population of set s, direction I; in the mixed units its deviation
+    // from the rest state (the double rest populations are added below)
+    auto pull = [&](int s, auto d) {
+        constexpr int I = decltype(d)::value;
+#if LBMK_MIXED
+        if (I == REST) return (Real)0;
+        return pull_dev(mc, v, a, s, I, p);
+#else
+        return pull_sf(mc, v, a, s, I, p);
+#endif
+    };
+    auto rest_part = [&](int s) {
+#if LBMK_MIXED
+        return mc.ref0[s] + v.rest()[(size_t)s * N + n];
+#else
+        (void)s;
+        return 0.0;
+#endif
+    };
+
+    // mixture set
+    double rho, P2[6];
+    Real js[3];
     {
-        double eu[6];
-        mixture_energy_poly<M>(mc, Y, eu);
-        T = solve_T(eu, sm.rhoE * ir - 0.5 * usq, a.macro[DR_T * N + n], a.status);
-        if (mc.transport) Cv = dpoly5(eu, T);
+        Real a0, P6[6];
+        row_moments<true, Real>([&](auto d) { return pull(M - 1, d); }, a0, js[0], js[1], js[2], P6);
+        rho = cvt<double>(a0);
+#if LBMK_MIXED
+        rho += rest_part(M - 1);
+#endif
+#pragma unroll
+        for (int k = 0; k < 6; ++k) P2[k] = cvt<double>(P6[k]);
+#if LBMK_MIXED
+#pragma unroll
+        for (int d = 0; d < 3; ++d) P2[d] += mc.refP[M - 1][d];
+#endif
     }
+    const double ir = 1.0 / rho;
+    const double u[3] = {cvt<double>(js[0]) * ir, cvt<double>(js[1]) * ir, cvt<double>(js[2]) * ir};
+    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+
+    // species densities and momenta; the last species is slaved (Eq. (strongest))
+    double rest = 0.0, inv_m = 0.0, eu[6];
+    bool neg = false;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) eu[k] = 0.0;
+#pragma unroll 1
+    for (int s = 0; s < M; ++s) {
+        double ra;
+        Real jx, jy, jz;
+        if (s < M - 1) {
+            Real a0;
+            row_moments<false, Real>([&](auto d) { return pull(s, d); }, a0, jx, jy, jz, nullptr);
+            ra = cvt<double>(a0);
+#if LBMK_MIXED
+            ra += rest_part(s);
+#endif
+            rest += ra;
+            js[0] -= jx;
+            js[1] -= jy;
+            js[2] -= jz;
+        } else {
+            ra = rho - rest;
+            jx = js[0];
+            jy = js[1];
+            jz = js[2];
+        }
+        Real *J = R + (size_t)(rr.du + 3 * s) * N + n;
+        J[0] = jx;
+        J[N] = jy;
+        J[2 * N] = jz;
+        const double Y = ra * ir;
+        inv_m = fma(Y, mc.invW[s], inv_m);
+        if (__double2hiint(ra) < 0)             // sign bit first: the compare only for negative values
+            neg |= ra < -1e-10 * rho;           // below rounding noise of trace species
+#pragma unroll
+        for (int k = 0; k < 6; ++k) eu[k] = fma(Y, mc.uco[s][k], eu[k]);
+        sh[s * bs] = ra;
+        sh[(M + s) * bs] = Y;
+        R[(size_t)(rr.y + s) * N + n] = cvt<Real>(Y);
+#if LBMK_MIXED
+        a.macro[(size_t)(dr_ra(M) + s) * N + n] = ra;
+#else
+        R[(size_t)(rr.ra + s) * N + n] = ra;
+#endif
+    }
+
+    // energy set
+    double rhoE, q[3];
+    row_moments<false, double>([&](auto d) { return pull_g(v, a, decltype(d)::value, p); }, rhoE, q[0], q[1], q[2],
+                               nullptr);
+    if (!(rho > 0.0) || !isfinite(rhoE)) flag(a.status, LBMK_BIT_NONFINITE);
+    if (neg) flag(a.status, LBMK_BIT_NEGATIVE);
+
+    // temperature, Eq. (temperature)
+    const double T = solve_T(eu, rhoE * ir - 0.5 * usq, a.macro[DR_T * N + n], a.status);
     const double Rm = mc.r_lat * inv_m;
     const double P = rho * Rm * T;
+    // enthalpies, Eq. (specHa); rest-direction equilibria of the species and
+    // mixture sets (Eqs. (feq), (feqmix))
+    double H = 0.0;
+#if LBMK_MIXED
+    const double c2[3] = {1.0 - u[0] * u[0], 1.0 - u[1] * u[1], 1.0 - u[2] * u[2]};
+#endif
+#pragma unroll 1
+    for (int s = 0; s < M; ++s) {
+        const double Ha = H_spec(mc, s, T);
+        H = fma(sh[(M + s) * bs], Ha, H);
+        R[(size_t)(rr.h + s) * N + n] = cvt<Real>(Ha);
+#if LBMK_MIXED
+        const double z = (s < M - 1 ? mc.Ra[s] : Rm) * T;
+        const double r = s < M - 1 ? sh[s * bs] : rho;
+        a.macro[(size_t)(DR_FEQ0 + s) * N + n] = r * (c2[0] - z) * (c2[1] - z) * (c2[2] - z);
+#endif
+    }
     // relaxation rates (Eqs. (mu), (lambda)) in the storage type: in the
     // mixed units they are stored and used as floats only; dfac scales the
     // binary diffusivities of mixture-averaged transport
     Real nup, nup1;
-    double dfac = 1.0;
+    double kappa = mc.r_lat * T / inv_m;        // Eq. (tauab): 1/tau_ab = kappa / (W_a W_b D_ab), kappa = m R_U T
     if (mc.transport) {
-        mixture_transport<M>(mc, Y, inv_m, T, P, Cv + Rm, nup, nup1, dfac);
+        double Y[M], dfac;
+#pragma unroll
+        for (int s = 0; s < M; ++s) Y[s] = sh[(M + s) * bs];
+        mixture_transport<M>(mc, Y, inv_m, T, P, dpoly5(eu, T) + Rm, nup, nup1, dfac);
+        kappa /= dfac;
     } else {
         nup = cvt<Real>(nu_prime(mc, Rm, T));
         nup1 = nup / cvt<Real>(mc.Pr);
@@ -1198,24 +1297,138 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd)
     const Real omega = (Real)1 / ((Real)0.5 + nup);
     const Real omega1 = (Real)1 / ((Real)0.5 + nup1);
 
-    // enthalpies, Eq. (specHa)
-    double Ha[M], H = 0.0;
-#pragma unroll
-    for (int s = 0; s < M; ++s) {
-        Ha[s] = H_spec(mc, s, T);
-        H = fma(Y[s], Ha[s], H);
-    }
+    // energy: equilibrium moments and the local part of
+    // Dq = (omega - omega_1)(q^* - q^eq) (Eqs. (gstareq1mom), (qdiff)) but
+    // for the diffusion velocities, added in k_diff; the grad-Y part
+    // (Eq. (corrFourier)) needs the neighbours and is added in k_step_g.
+    double qeq[3], Rt[6], tr3;
+    energy_moments(rho, u, P, H + 0.5 * usq, rhoE, qeq, Rt, tr3);
+    const double dP[6] = {P2[0] - (P + rho * u[0] * u[0]), P2[1] - (P + rho * u[1] * u[1]),
+                          P2[2] - (P + rho * u[2] * u[2]), P2[3] - rho * u[0] * u[1],
+                          P2[4] - rho * u[0] * u[2], P2[5] - rho * u[1] * u[2]};
+    const double uP[3] = {u[0] * dP[0] + u[1] * dP[3] + u[2] * dP[4], u[0] * dP[3] + u[1] * dP[1] + u[2] * dP[5],
+                          u[0] * dP[4] + u[1] * dP[5] + u[2] * dP[2]};
 
-    // Eq. (tauab): 1/tau_ab = kappa / (W_a W_b D_ab), kappa = m R_U T;
-    // 1/tau_a = sum_b Y_b / tau_ab.  From here to the diffusion velocities
-    // the arithmetic is in SReal: double, or float in the fast mixed unit
+    // the record: double rows
+    a.macro[DR_T * N + n] = T;
+    a.macro[(size_t)dr_ge(M) * N + n] = rhoE;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) a.macro[(size_t)(dr_gq(M) + d) * N + n] = qeq[d];
+#pragma unroll
+    for (int d = 0; d < 6; ++d) a.macro[(size_t)(dr_gr(M) + d) * N + n] = Rt[d];
+    a.macro[(size_t)dr_gtr(M) * N + n] = tr3;
+#if LBMK_MIXED
+#pragma unroll
+    for (int d = 0; d < 3; ++d) a.macro[(size_t)(dr_u(M) + d) * N + n] = u[d];
+    a.macro[(size_t)dr_hk(M) * N + n] = LBMK_FAST ? ir : 0.5 * kappa * ir;
+#endif
+    // storage-type rows
+    R[(size_t)rr.nup * N + n] = nup;
+    // Phi (Eq. (Xalpha)), stored in the storage type and formed in it
+    const Real rhoR = cvt<Real>(rho), rtR = cvt<Real>(Rm * T), ph = (Real)1 - (Real)3 * rtR;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const Real ud = cvt<Real>(u[d]);
+        R[(size_t)(rr.phi + d) * N + n] = rhoR * ud * (ph - ud * ud);
+        R[(size_t)(rr.u + d) * N + n] = ud;
+        // the difference is formed in double (it cancels), the product in the storage type
+        R[(size_t)(rr.dq + d) * N + n] = (omega - omega1) * cvt<Real>(q[d] - uP[d] - qeq[d]);
+    }
+    R[(size_t)rr.rho * N + n] = rhoR;
+    R[(size_t)rr.kappa * N + n] = cvt<Real>(kappa);
+    R[(size_t)rr.rt * N + n] = rtR;
+    R[(size_t)rr.om * N + n] = omega;
+    R[(size_t)rr.om1 * N + n] = omega1;
+    R[(size_t)rr.p * N + n] = cvt<Real>(P);
+}
+
+extern __shared__ double sh_pre[];
+
+template <int M>
+__global__ void __launch_bounds__(LBMK_BLOCK, LBMK_PRE_MINB) k_pre(StepArgs a)
+{
+    Node nd;
+    if (!node_of(nd, a)) return;
+    pre_node<M>(a, nd, sh_pre + threadIdx.x, blockDim.x);
+}
+
+// ---------------------------------------------------------------------
+// Pass 1b: Stefan-Maxwell diffusion velocities (Eq. (transform1)), beta_a
+// and their part of Dq.
+// FX: the tables are in the range of the fixed-point sums (MechConst::
+// mix_fixed); sh: this thread's shared memory, diff_cols<M, FX>() columns
+// of bs doubles.
+// ---------------------------------------------------------------------
+
+// Whether the Stefan-Maxwell solve refines a float factorisation
+// (lbm_diffusion.cuh): in the mixed unit, whose velocities are stored as
+// floats, from four species on.  (In the fast mixed unit the whole solve is
+// in float; with two or three species the LDL^T solve is cheaper.)
+template <int M, bool FX>
+constexpr bool kRefined = FX && M >= 4 && LBMK_MIXED && !LBMK_FAST;
+
+template <int M, bool FX>
+constexpr int diff_cols() { return kRefined<M, FX> ? 2 * M : 0; }
+
+template <int M, bool FX>
+__device__ __forceinline__ void diff_node(const StepArgs &a, const Node &nd, double *sh, int bs)
+{
+    const MechConst &mc = c_mech[a.slot];
+    const int n = nd.n;
+    const size_t N = a.N;
+    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    Real *R = rec(a);
+    auto ld = [&](int row) { return R[(size_t)row * N + n]; };
+    Real duR[M][3], itaR[M];
+#if LBMK_MIXED && !LBMK_FAST
+    if constexpr (kRefined<M, FX>) {
+        bool bad = false;
+        diffusion_refined<M>(mc, a.macro + (size_t)dr_ra(M) * N + n, a.macro + (size_t)dr_u(M) * N + n,
+                             R + (size_t)rr.du * N + n, N, a.macro[(size_t)dr_hk(M) * N + n], sh, bs, duR, itaR, &bad);
+        if (bad) flag(a.status, LBMK_BIT_PIVOT);
+    } else
+#endif
+    {
+    // The arithmetic is in SReal: double, or float in the fast mixed unit
     // (the results are stored as floats there, and the solve below is well
     // conditioned: B is diagonally dominant after the symmetric scaling by Y).
-    const double kappa = mc.transport ? mc.r_lat * T / (inv_m * dfac) : mc.r_lat * T / inv_m;
-    const SReal kap = cvt<SReal>(kappa), irr = cvt<SReal>(ir);
-    SReal Yr[M], ur[3] = {cvt<SReal>(u[0]), cvt<SReal>(u[1]), cvt<SReal>(u[2])};
+    SReal Yr[M], ur[3], irr, kap;
+    Real ja[M][3];
+    {
+#if LBMK_MIXED
+        const double *ra = a.macro + (size_t)dr_ra(M) * N + n;
 #pragma unroll
-    for (int s = 0; s < M; ++s) Yr[s] = cvt<SReal>(Y[s]);
+        for (int d = 0; d < 3; ++d) ur[d] = cvt<SReal>(a.macro[(size_t)(dr_u(M) + d) * N + n]);
+#else
+        const double *ra = R + (size_t)rr.ra * N + n;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) ur[d] = ld(rr.u + d);
+#endif
+#if LBMK_FAST
+        irr = cvt<SReal>(a.macro[(size_t)dr_hk(M) * N + n]);
+        kap = ld(rr.kappa);
+#pragma unroll
+        for (int s = 0; s < M; ++s) Yr[s] = ld(rr.y + s);
+        (void)ra;
+#else
+        double rho = 0.0;
+#pragma unroll
+        for (int s = 0; s < M; ++s) rho += ra[(size_t)s * N];
+        irr = 1.0 / rho;
+#if LBMK_MIXED
+        kap = 2.0 * a.macro[(size_t)dr_hk(M) * N + n] * rho;
+#else
+        kap = ld(rr.kappa);
+#endif
+#pragma unroll
+        for (int s = 0; s < M; ++s) Yr[s] = ra[(size_t)s * N] * irr;
+#endif
+#pragma unroll
+        for (int s = 0; s < M; ++s)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) ja[s][d] = ld(rr.du + 3 * s + d);
+    }
+    // 1/tau_a = sum_b Y_b / tau_ab
     SReal ita[M];
 #pragma unroll
     for (int s = 0; s < M; ++s) {
@@ -1288,101 +1501,39 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd)
                 du[i][d] = sacc;
             }
     }
-
-    // energy: equilibrium moments and the local part of
-    // Dq = (omega - omega_1)(q^* - q^eq) (Eqs. (gstareq1mom), (qdiff)); the
-    // grad-Y part (Eq. (corrFourier)) needs the neighbours and is added in k_step.
-    const double hk = H + 0.5 * usq;
-    double qeq[3], Rt[6], tr3;
-    energy_moments(rho, u, P, hk, sm.rhoE, qeq, Rt, tr3);
-    Real dq[3], HaR[M], YR[M], duR[M][3];
-    {
-        const double dP[6] = {sm.P[0] - (P + rho * u[0] * u[0]), sm.P[1] - (P + rho * u[1] * u[1]),
-                              sm.P[2] - (P + rho * u[2] * u[2]), sm.P[3] - rho * u[0] * u[1],
-                              sm.P[4] - rho * u[0] * u[2], sm.P[5] - rho * u[1] * u[2]};
-        const double uP[3] = {u[0] * dP[0] + u[1] * dP[3] + u[2] * dP[4],
-                              u[0] * dP[3] + u[1] * dP[1] + u[2] * dP[5],
-                              u[0] * dP[4] + u[1] * dP[5] + u[2] * dP[2]};
-        // Dq is stored in the storage type: the differences are formed in
-        // double (they cancel), the products with the stored values of
-        // omega, omega_1, H_a, Y_a and du_a in the storage type
-        Real HY[M];
-#pragma unroll
-        for (int s = 0; s < M; ++s) {
-            HaR[s] = cvt<Real>(Ha[s]);
-            YR[s] = cvt<Real>(Yr[s]);
-            HY[s] = HaR[s] * YR[s];
-#pragma unroll
-            for (int d = 0; d < 3; ++d) duR[s][d] = cvt<Real>(du[s][d]);
-        }
-        const Real orho = omega1 * cvt<Real>(rho);
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            Real hyd = 0;
-#pragma unroll
-            for (int s = 0; s < M; ++s) hyd = fma(HY[s], duR[s][d], hyd);
-            dq[d] = (omega - omega1) * cvt<Real>(sm.q[d] - uP[d] - qeq[d]) + orho * hyd;
-        }
-    }
-
-    // the record: double rows
-    a.macro[DR_T * N + n] = T;
-    a.macro[(size_t)dr_ge(M) * N + n] = sm.rhoE;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) a.macro[(size_t)(dr_gq(M) + d) * N + n] = qeq[d];
-#pragma unroll
-    for (int d = 0; d < 6; ++d) a.macro[(size_t)(dr_gr(M) + d) * N + n] = Rt[d];
-    a.macro[(size_t)dr_gtr(M) * N + n] = tr3;
-#if LBMK_MIXED
-    // rest-direction equilibria of the species and mixture sets (Eqs. (feq), (feqmix))
-    {
-        const double c2[3] = {1.0 - u[0] * u[0], 1.0 - u[1] * u[1], 1.0 - u[2] * u[2]};
-#pragma unroll
-        for (int s = 0; s < M; ++s) {
-            const double z = (s < M - 1 ? mc.Ra[s] : Rm) * T;
-            const double r = s < M - 1 ? rho_a[s] : rho;
-            a.macro[(size_t)(DR_FEQ0 + s) * N + n] = r * (c2[0] - z) * (c2[1] - z) * (c2[2] - z);
-        }
-    }
-#endif
-    // storage-type rows
-    const RecRows rr = rec_rows(M);
-    Real *R = rec(a);
-    R[(size_t)rr.nup * N + n] = nup;
-    // Phi (Eq. (Xalpha)), stored in the storage type and formed in it
-    const Real rhoR = cvt<Real>(rho), rtR = cvt<Real>(Rm * T), ph = (Real)1 - (Real)3 * rtR;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const Real ud = cvt<Real>(ur[d]);
-        R[(size_t)(rr.phi + d) * N + n] = rhoR * ud * (ph - ud * ud);
-        R[(size_t)(rr.u + d) * N + n] = ud;
-        R[(size_t)(rr.dq + d) * N + n] = dq[d];
-    }
 #pragma unroll
     for (int s = 0; s < M; ++s) {
-        R[(size_t)(rr.y + s) * N + n] = YR[s];
+        itaR[s] = cvt<Real>(ita[s]);
 #pragma unroll
-        for (int d = 0; d < 3; ++d) R[(size_t)(rr.du + 3 * s + d) * N + n] = duR[s][d];
+        for (int d = 0; d < 3; ++d) duR[s][d] = cvt<Real>(du[s][d]);
+    }
+    }
+    // Dq: + omega_1 rho sum_a H_a Y_a du_a, in the storage type
+    Real hyd[3] = {0, 0, 0};
+#pragma unroll
+    for (int s = 0; s < M; ++s) {
+        const Real HY = ld(rr.h + s) * ld(rr.y + s);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            hyd[d] = fma(HY, duR[s][d], hyd[d]);
+            R[(size_t)(rr.du + 3 * s + d) * N + n] = duR[s][d];
+        }
         // beta_a = 1/(2 tau_a + 1), Eq. (fStar): a parameter of the species
         // collision, formed in the storage type it is used in
-        const Real it = cvt<Real>(ita[s]);
-        R[(size_t)(rr.beta + s) * N + n] = it / ((Real)2 + it);
-        R[(size_t)(rr.h + s) * N + n] = HaR[s];
+        R[(size_t)(rr.beta + s) * N + n] = itaR[s] / ((Real)2 + itaR[s]);
     }
-    R[(size_t)rr.rho * N + n] = rhoR;
-    R[(size_t)rr.kappa * N + n] = cvt<Real>(kap);
-    R[(size_t)rr.rt * N + n] = rtR;
-    R[(size_t)rr.om * N + n] = omega;
-    R[(size_t)rr.om1 * N + n] = omega1;
-    R[(size_t)rr.p * N + n] = cvt<Real>(P);
+    const Real orho = ld(rr.om1) * ld(rr.rho);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) R[(size_t)(rr.dq + d) * N + n] = fma(orho, hyd[d], ld(rr.dq + d));
 }
 
-template <int M>
-__global__ void __launch_bounds__(LBMK_BLOCK, LBMK_PRE_MINB) k_pre(StepArgs a)
+template <int M, bool FX>
+__global__ void __launch_bounds__(LBMK_BLOCK, LBMK_DIFF_MINB) k_diff(StepArgs a)
 {
     Node nd;
-    if (!node_of(nd, a)) return;
-    pre_node<M>(a, nd);
+    nd.n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (nd.n >= a.N) return;
+    diff_node<M, FX>(a, nd, sh_pre + threadIdx.x, blockDim.x);
 }
 
 // ---------------------------------------------------------------------
@@ -1393,7 +1544,7 @@ template <int M>
 __device__ __forceinline__ void grad_node(const StepArgs &a, const Node &nd)
 {
     const size_t N = a.N;
-    const RecRows rr = rec_rows(M);
+    const RecRows rr = rec_rows(M, LBMK_MIXED);
     Real *R = rec(a);
     const Real *Phi = R + (size_t)rr.phi * N;
     StencilIdx st;
@@ -1436,7 +1587,7 @@ __device__ __forceinline__ void collide_energy(const StepArgs &a, const Node &nd
 {
     const int n = nd.n;
     const size_t N = a.N;
-    const RecRows rr = rec_rows(M);
+    const RecRows rr = rec_rows(M, LBMK_MIXED);
     const Real *R = rec(a);
     auto ld = [&](int row) { return R[(size_t)row * N + n]; };
     auto ldd = [&](int row) { return a.macro[(size_t)row * N + n]; };
@@ -1540,7 +1691,7 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
     const MechConst &mc = c_mech[a.slot];
     const int n = nd.n;
     const size_t N = a.N;
-    const RecRows rr = rec_rows(M);
+    const RecRows rr = rec_rows(M, LBMK_MIXED);
     const Real *R = rec(a);
     auto ld = [&](int row) { return R[(size_t)row * N + n]; };
     auto ldd = [&](int row) { return a.macro[(size_t)row * N + n]; };
@@ -1772,7 +1923,15 @@ int launch_one(const StepArgs &a, int k)
             k_ghost<M><<<grid_for(2 * (a.nseg > 1 ? a.nseg : 1) * plane), LBMK_BLOCK, 0, a.stream>>>(a);
         }
         break;
-    case LBMK_K_PRE: k_pre<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
+    case LBMK_K_PRE: {
+        k_pre<M><<<grid_for(a.N, bs), bs, pre_cols<M>() * bs * sizeof(double), a.stream>>>(a);
+        constexpr bool FX = kRefined<M, true>;
+        if (FX && a.fixed)
+            k_diff<M, FX><<<grid_for(a.N, bs), bs, diff_cols<M, FX>() * bs * sizeof(double), a.stream>>>(a);
+        else
+            k_diff<M, false><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a);
+        break;
+    }
     case LBMK_K_CHEM: break;            // the rates are formed inside k_step
     case LBMK_K_GRAD: k_grad<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
     case LBMK_K_STEPG: k_step_g<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
@@ -1856,7 +2015,7 @@ __device__ __forceinline__ void tile_loop(const StepArgs &a, int chunk, unsigned
 }
 
 // One time step of the persistent kernel over the buffers of b.
-template <int M>
+template <int M, bool FX>
 __device__ __forceinline__ bool persist_step(const StepArgs &b, int tile, GridBarrier *bar, unsigned nb, unsigned cap)
 {
     if (b.bc_x == 1) {
@@ -1864,7 +2023,10 @@ __device__ __forceinline__ bool persist_step(const StepArgs &b, int tile, GridBa
         for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x) ghost_node<M>(b, g);
         if (!grid_barrier(bar, nb, cap, b.status)) return false;
     }
-    tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) { pre_node<M>(b, nd); });
+    tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) {
+        pre_node<M>(b, nd, sh_step + threadIdx.x, LBMK_BLOCK);
+        diff_node<M, FX>(b, nd, sh_step + threadIdx.x, LBMK_BLOCK);
+    });
     if (!grid_barrier(bar, nb, cap, b.status)) return false;
     tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) { grad_node<M>(b, nd); });
     if (!grid_barrier(bar, nb, cap, b.status)) return false;
@@ -1880,26 +2042,26 @@ __device__ __forceinline__ bool persist_step(const StepArgs &b, int tile, GridBa
 // a0 steps src -> dst, a1 the same with the buffers swapped: the steps
 // alternate between the two parameter blocks, which the phases then read
 // in place (no per-step copy of the arguments)
-template <int M>
+template <int M, bool FX>
 __global__ void __launch_bounds__(LBMK_BLOCK, LBMK_PRE_MINB) k_persist(StepArgs a0, StepArgs a1, int nsteps, int tile,
                                                                       GridBarrier *bar, unsigned cap)
 {
     const unsigned nb = gridDim.x;
     for (int t = 0; t < nsteps; t += 2) {
-        if (!persist_step<M>(a0, tile, bar, nb, cap)) return;
-        if (t + 1 < nsteps && !persist_step<M>(a1, tile, bar, nb, cap)) return;
+        if (!persist_step<M, FX>(a0, tile, bar, nb, cap)) return;
+        if (t + 1 < nsteps && !persist_step<M, FX>(a1, tile, bar, nb, cap)) return;
     }
 }
 
-template <int M>
-int run_persistent(const StepArgs &a, int nsteps, int tile_mult, GridBarrier *bar, unsigned cap)
+template <int M, bool FX>
+int launch_persistent(const StepArgs &a, int nsteps, int tile_mult, GridBarrier *bar, unsigned cap)
 {
     if (nsteps < 1 || tile_mult < 1) return (int)cudaErrorInvalidValue;
     int per_sm = 0, dev = 0, nsm = 0;
     static std::atomic<unsigned long long> opted{0};
-    const int eo = opt_in_smem(k_persist<M>, step_smem<M>(LBMK_BLOCK), opted);
+    const int eo = opt_in_smem(k_persist<M, FX>, step_smem<M>(LBMK_BLOCK), opted);
     if (eo) return eo;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_persist<M>, LBMK_BLOCK,
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_persist<M, FX>, LBMK_BLOCK,
                                                                   step_smem<M>(LBMK_BLOCK));
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -1915,8 +2077,15 @@ int run_persistent(const StepArgs &a, int nsteps, int tile_mult, GridBarrier *ba
     GridBarrier *bb = bar;
     unsigned cc = cap;
     void *args[] = {(void *)&a0, (void *)&a1, (void *)&ns, (void *)&tl, (void *)&bb, (void *)&cc};
-    return (int)cudaLaunchCooperativeKernel((const void *)k_persist<M>, dim3(blocks), dim3(LBMK_BLOCK), args,
+    return (int)cudaLaunchCooperativeKernel((const void *)k_persist<M, FX>, dim3(blocks), dim3(LBMK_BLOCK), args,
                                             step_smem<M>(LBMK_BLOCK), a.stream);
+}
+template <int M>
+int run_persistent(const StepArgs &a, int nsteps, int tile_mult, GridBarrier *bar, unsigned cap)
+{
+    if (kRefined<M, true> && a.fixed)
+        return launch_persistent<M, kRefined<M, true>>(a, nsteps, tile_mult, bar, cap);
+    return launch_persistent<M, false>(a, nsteps, tile_mult, bar, cap);
 }
 #endif  // LBMK_COHERENT_LOADS
 
@@ -2473,7 +2642,7 @@ __global__ void __launch_bounds__(LBMK_BLOCK) k_flame1(StepArgs a, double *scr)
     if (!node_of(nd, a)) return;
     const size_t N = a.N;
     const int n = nd.n;
-    const RecRows rr = rec_rows(M);
+    const RecRows rr = rec_rows(M, LBMK_MIXED);
     const Real *R = rec(a);
     const double *Tr = a.macro + (size_t)DR_T * N;
     StencilIdx st;
@@ -2508,7 +2677,7 @@ __global__ void __launch_bounds__(LBMK_HRR_THREADS) k_flame2(StepArgs a, const d
     if (!node_of(nd, a)) return;
     const size_t N = a.N;
     const int n = nd.n;
-    const RecRows rr = rec_rows(M);
+    const RecRows rr = rec_rows(M, LBMK_MIXED);
     const Real *R = rec(a);
     StencilIdx st;
     make_stencil(st, nd, a);

@@ -70,9 +70,11 @@ static inline int lbm_pack_tables(const lbm_species *sp, const lbm_mechanism *me
             mc.inv_WWD_f[a][b] = (float)mc.inv_WWD[a][b];
         }
     }
-    // Fixed-point 1/D_ab for the cross terms of the double collision: the
-    // largest entry keeps its leading bit at 2^57, so that entries down to
-    // 1/32 of it keep all 53 bits; wider ranges take the floating sums.
+    // Fixed-point 1/D_ab for the sums over the species: the largest entry
+    // keeps its leading bit at 2^57, so that entries down to 1/32 of it keep
+    // all 53 bits.  Wider ranges, and magnitudes of 1/D and W so far from
+    // one that the float scales of lbm_diffusion.cuh could leave their
+    // normal range, take the floating sums.
     {
         double top = 0.0, low = INFINITY;
         for (int a = 0; a < M; ++a)
@@ -82,7 +84,12 @@ static inline int lbm_pack_tables(const lbm_species *sp, const lbm_mechanism *me
                     low = fmin(low, 1.0 / sp->D[M * a + b]);
                 }
         const int e = isfinite(top) ? ilogb(top) : 0;
-        mc.mix_fixed = isfinite(top) && top <= 32.0 * low && e > -500 && e < 500;
+        mc.mix_fixed = M <= LBMK_MIXM && isfinite(top) && top <= 32.0 * low && e >= -12 && e <= 20;
+        for (int a = 0; a < M; ++a) {
+            if (sp->W[a] < 0x1p-12 || sp->W[a] > 0x1p+12) mc.mix_fixed = 0;
+            mc.invW_h[a] = (float)mc.invW[a];
+            mc.invW_l[a] = (float)(mc.invW[a] - (double)mc.invW_h[a]);
+        }
         mc.mix_exp = e - 57;
         for (int a = 0; a < M && mc.mix_fixed; ++a)
             for (int b = 0; b < M; ++b)
@@ -90,6 +97,8 @@ static inline int lbm_pack_tables(const lbm_species *sp, const lbm_mechanism *me
                     const long long v = (long long)ldexp(1.0 / sp->D[M * a + b], 57 - e);
                     mc.mixh[a][b] = (int)(v >> 29);
                     mc.mixl[a][b] = (int)(v & 0x1fffffff);
+                    mc.invD_h[a][b] = (float)(1.0 / sp->D[M * a + b]);
+                    mc.invD_l[a][b] = (float)(1.0 / sp->D[M * a + b] - (double)mc.invD_h[a][b]);
                 }
     }
     mc.transport = sp->transport;
