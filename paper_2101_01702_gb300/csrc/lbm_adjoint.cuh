@@ -341,20 +341,12 @@ __device__ void adj_collide_node(const MechConst &mc, const StepArgs &a, const A
     const PopView v = view(a.src, a);
     double rho_a[M], ja[M][3];
     Sums sm;
-    pull_moments<M, true>(mc, a, p, n, rho_a, ja, sm);
+    pull_moments<M, true>(mc, a, p, n, sm, [&](int s, double ra, const double *j) {
+        rho_a[s] = ra;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) ja[s][d] = j[d];
+    });
     const double rho = sm.rho, ir = 1.0 / rho;
-    {
-        double rest = 0.0, js[3] = {sm.j[0], sm.j[1], sm.j[2]};
-#pragma unroll
-        for (int s = 0; s < M - 1; ++s) {
-            rest += rho_a[s];
-#pragma unroll
-            for (int d = 0; d < 3; ++d) js[d] -= ja[s][d];
-        }
-        rho_a[M - 1] = rho - rest;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) ja[M - 1][d] = js[d];
-    }
     double Y[M], inv_m = 0.0;
 #pragma unroll
     for (int s = 0; s < M; ++s) {

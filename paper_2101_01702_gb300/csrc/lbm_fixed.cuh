@@ -24,14 +24,19 @@ __device__ __forceinline__ int biased_exponent(double d) { return (__double2hiin
 // d in units of 2^(e - 1080), for e at least d's biased exponent: the
 // largest operand of a block keeps its leading bit at 2^57; bits below
 // the unit are dropped.
-__device__ __forceinline__ Limbs58 to_limbs58(double d, int e)
+__device__ __forceinline__ long long to_fixed58(double d, int e)
 {
     const int hi = __double2hiint(d), ed = (hi >> 20) & 0x7ff;
     const unsigned mh = ((unsigned)hi & 0xfffffu) | (ed ? 0x100000u : 0u);
     const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << 5;
     const int sh = e - ed < 63 ? e - ed : 63;                 // m < 2^58
-    long long v = (long long)(m >> sh);
-    v = hi < 0 ? -v : v;
+    const long long v = (long long)(m >> sh);
+    return hi < 0 ? -v : v;
+}
+
+__device__ __forceinline__ Limbs58 to_limbs58(double d, int e)
+{
+    const long long v = to_fixed58(d, e);
     return Limbs58{(int)(v >> 29), (int)((unsigned)v & 0x1fffffffu)};
 }
 

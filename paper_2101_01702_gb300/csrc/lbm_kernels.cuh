@@ -332,10 +332,12 @@ struct Src {
     size_t idx;
 };
 
+// GH false: for a node none of whose pulls reaches a ghost plane.
+template <bool GH = true>
 __device__ __forceinline__ Src src_of(int i, const PullIdx &p, const StepArgs &a)
 {
     const int xs = p.xs[CX(i) + 1];
-    const int gp = p.gp[CX(i) + 1];
+    const int gp = GH ? p.gp[CX(i) + 1] : -1;
     const int yz = p.yz[(CY(i) + 1) + 3 * (CZ(i) + 1)];
     if (gp >= 0) {
         const int nlat = a.nseg > 1 ? a.nseg : 1;
@@ -354,16 +356,18 @@ __device__ __forceinline__ double load_ghost(const StepArgs &a, int plane_idx, i
                  yz);
 }
 
+template <bool GH = true>
 __device__ __forceinline__ Real pull_sf(const MechConst &mc, const PopView &v, const StepArgs &a, int s, int i,
                                         const PullIdx &p)
 {
-    const Src sr = src_of(i, p, a);
+    const Src sr = src_of<GH>(i, p, a);
     return sr.ghost ? (Real)load_ghost(a, sr.side, s, i, sr.idx) : load_sf(mc, v, s, i, sr.idx);
 }
 
+template <bool GH = true>
 __device__ __forceinline__ double pull_g(const PopView &v, const StepArgs &a, int i, const PullIdx &p)
 {
-    const Src sr = src_of(i, p, a);
+    const Src sr = src_of<GH>(i, p, a);
     return sr.ghost ? load_ghost(a, sr.side, a.M, i, sr.idx) : load_g(v, i, sr.idx);
 }
 
@@ -457,20 +461,22 @@ __device__ __forceinline__ double dpoly5(const double u[6], double T)
     return fma(fma(fma(fma(5.0 * u[5], T, 4.0 * u[4]), T, 3.0 * u[3]), T, 2.0 * u[2]), T, u[1]);
 }
 
-// Newton iteration on U(T) = e from T.  It stops once a correction is at
-// most 1e-7 T: Newton's error after that step is about (C_v'/2C_v) dT^2,
-// below 1e-13 T for these polynomials (C_v'/C_v is of order 1/T), so the
-// further iteration a 1e-13 test would take changes T by less than that.
+// Newton iteration on U(T) = e from T.  The residual is formed in double;
+// the derivative and the quotient, which only scale the correction, in float
+// (a float division and conversions on the integer pipe in place of 13
+// FP64 operations per iteration).  It stops once a correction is at most
+// 5e-10 T: the error left is then the correction's relative error, 2e-7, of
+// that and Newton's quadratic term, (C_v'/2C_v) dT^2: 1e-16 T in all.
 __device__ __forceinline__ double solve_T(const double u[6], double e, double T, unsigned *status)
 {
-    const double d5 = 5.0 * u[5], d4 = 4.0 * u[4], d3 = 3.0 * u[3], d2 = 2.0 * u[2];   // C_v's coefficients
+    const float d5 = 5.0f * d2f(u[5]), d4 = 4.0f * d2f(u[4]), d3 = 3.0f * d2f(u[3]), d2 = 2.0f * d2f(u[2]),
+                d1 = d2f(u[1]);                               // C_v's coefficients
     for (int it = 0; it < 50; ++it) {
-        const double F = poly5(u, T) - e;
-        const double Fp = fma(fma(fma(fma(d5, T, d4), T, d3), T, d2), T, u[1]);
-        const double dT = F / Fp;
-        T -= dT;
+        const float t = d2f(T);
+        const float dT = d2f(poly5(u, T) - e) / fma(fma(fma(fma(d5, t, d4), t, d3), t, d2), t, d1);
+        T -= f2d(dT);
         if (!finite_bits(T)) { flag(status, LBMK_BIT_NONFINITE); return T; }
-        if (fabs(dT) <= 1e-7 * fabs(T)) return T;
+        if (fabsf(dT) <= 5e-10f * fabsf(t)) return T;
     }
     flag(status, LBMK_BIT_NEWTON);
     return T;
@@ -697,75 +703,125 @@ __device__ __forceinline__ void row_moments(LD &&ld, V &s0, V &sx, V &sy, V &sz,
     });
 }
 
-// Moments of the pulled populations.  Species a < M-1 give rho_a and j_a;
-// f gives rho, j and (WITH_P) the pressure tensor; g gives rho E and q.
-struct Sums {
-    double rho, j[3], P[6], rhoE, q[3];   // P: xx, yy, zz, xy, xz, yz
-    Real jr[3];                           // j as summed, in the storage type
-};
+// The same sums of 27 doubles on the integer pipe: the moving populations are
+// brought to the largest one's exponent (to 2^-57 of it) and added as
+// integers, each sum rounded once; the rest population, up to a thousand
+// times larger and part of the zeroth moment alone, is added in double.  57
+// (94 with WITH_P) FP64 additions, 76 cycles of a scheduler each, become
+// about 600 (700) integer instructions.  What is dropped is below 2^-57 of
+// the largest moving population from each, downwards from all of one sign,
+// so that most of it cancels in the first moments.
+template <bool WITH_P, class LD>
+__device__ __forceinline__ void fixed_row_moments(LD &&ld, double &s0, double &sx, double &sy, double &sz, double *P6)
+{
+    double v[LBMK_Q];
+    int e = 0;
+    for_dirs<0, LBMK_Q>([&](auto d) {
+        constexpr int I = decltype(d)::value;
+        v[I] = ld(d);
+        if constexpr (I != REST) e = max(e, biased_exponent(v[I]));
+    });
+    long long t0, tx, ty, tz, tP[6];
+    row_moments<WITH_P, long long>([&](auto d) {
+        constexpr int I = decltype(d)::value;
+        return I == REST ? 0ll : to_fixed58(v[I], e);
+    }, t0, tx, ty, tz, tP);
+    const bool nan = e == 0x7ff;                           // an infinite or NaN population
+    auto out = [&](long long x) {
+        return nan ? __longlong_as_double(0x7ff8000000000000ll) : double_of_int64(x, e - 1080);
+    };
+    s0 = out(t0) + v[REST];
+    sx = out(tx);
+    sy = out(ty);
+    sz = out(tz);
+    if constexpr (WITH_P)
+#pragma unroll
+        for (int k = 0; k < 6; ++k) P6[k] = out(tP[k]);
+}
 
 // In the mixed units the moving populations are summed as the stored float
 // deviations from the set's rest state; its moments (ref0, refP: double,
 // the first moments vanish) and the double rest population are added once.
 #if LBMK_MIXED
+template <bool GH>
 __device__ __forceinline__ Real pull_dev(const MechConst &mc, const PopView &v, const StepArgs &a, int s, int i,
                                          const PullIdx &p)
 {
-    const Src sr = src_of(i, p, a);
+    const Src sr = src_of<GH>(i, p, a);
     return sr.ghost ? (Real)load_ghost(a, sr.side, s, i, sr.idx) - RAWREF(s, i) : load_raw_sf(v, s, i, sr.idx);
 }
 #endif
 
-template <int M, bool WITH_P>
-__device__ __forceinline__ void pull_moments(const MechConst &mc, const StepArgs &a, const PullIdx &p, int n,
-                                             double *rho_a, Real (*ja)[3], Sums &sm)
+// Zeroth and first moments (and with WITH_P the second) of species or
+// mixture set s < M; the first as summed, in the storage type.
+template <bool WITH_P, bool GH>
+__device__ __forceinline__ void set_moments(const MechConst &mc, const PopView &v, const StepArgs &a, const PullIdx &p,
+                                            int n, int s, double &r, Real *j, double *P)
 {
-    const PopView v = view(a.src, a);
-#pragma unroll
-    for (int s = 0; s < M - 1; ++s) {
-        Real a0, ax, ay, az;
-        row_moments<false, Real>([&](auto d) {
-            constexpr int I = decltype(d)::value;
 #if LBMK_MIXED
-            if (I == REST) return (Real)0;                    // the double rest population: below
-            return pull_dev(mc, v, a, s, I, p);
-#else
-            return pull_sf(mc, v, a, s, I, p);
-#endif
-        }, a0, ax, ay, az, nullptr);
-        rho_a[s] = cvt<double>(a0);
-#if LBMK_MIXED
-        rho_a[s] += mc.ref0[s] + v.rest()[(size_t)s * a.N + n];
-#endif
-        ja[s][0] = ax;
-        ja[s][1] = ay;
-        ja[s][2] = az;
-    }
-    double g0, qx, qy, qz;
-    row_moments<false, double>([&](auto d) { return pull_g(v, a, decltype(d)::value, p); }, g0, qx, qy, qz, nullptr);
-    Real a0, ax, ay, az, P6[6];
+    Real a0, P6[6];
     row_moments<WITH_P, Real>([&](auto d) {
         constexpr int I = decltype(d)::value;
-#if LBMK_MIXED
-        if (I == REST) return (Real)0;
-        return pull_dev(mc, v, a, M - 1, I, p);
-#else
-        return pull_sf(mc, v, a, M - 1, I, p);
-#endif
-    }, a0, ax, ay, az, P6);
-    sm.rho = cvt<double>(a0);
-    sm.rhoE = g0;
-    sm.jr[0] = ax; sm.jr[1] = ay; sm.jr[2] = az;
-    sm.j[0] = cvt<double>(ax); sm.j[1] = cvt<double>(ay); sm.j[2] = cvt<double>(az);
-    sm.q[0] = qx; sm.q[1] = qy; sm.q[2] = qz;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) sm.P[k] = WITH_P ? cvt<double>(P6[k]) : 0.0;
-#if LBMK_MIXED
-    sm.rho += mc.ref0[M - 1] + v.rest()[(size_t)(M - 1) * a.N + n];
+        return I == REST ? (Real)0 : pull_dev<GH>(mc, v, a, s, I, p);           // the double rest population: below
+    }, a0, j[0], j[1], j[2], P6);
+    r = cvt<double>(a0) + (mc.ref0[s] + v.rest()[(size_t)s * v.N + n]);
     if constexpr (WITH_P)
 #pragma unroll
-        for (int d = 0; d < 3; ++d) sm.P[d] += mc.refP[M - 1][d];
+        for (int k = 0; k < 6; ++k) P[k] = cvt<double>(P6[k]) + (k < 3 ? mc.refP[s][k] : 0.0);
+#else
+    (void)n;
+    fixed_row_moments<WITH_P>([&](auto d) { return pull_sf<GH>(mc, v, a, s, decltype(d)::value, p); }, r, j[0], j[1], j[2],
+                              P);
 #endif
+}
+
+// Moments of the pulled populations of a node: the mixture set gives rho,
+// rho u and (WITH_P) the pressure tensor, the energy set rho E and q, and
+// each species its density and momentum, the last one slaved (Eq.
+// (strongest)), handed to put(s, rho_a, j_a) in order after rho and rho u
+// are known (in sm).  The loop over the species is not unrolled, see
+// pre_node.
+struct Sums {
+    double rho, j[3], P[6], rhoE, q[3];   // P: xx, yy, zz, xy, xz, yz
+};
+
+template <int M, bool WITH_P, class Put>
+__device__ __forceinline__ void pull_moments(const MechConst &mc, const StepArgs &a, const PullIdx &p, int n, Sums &sm,
+                                             Put &&put)
+{
+    const PopView v = view(a.src, a);
+    // nodes away from the x faces of a lattice take code without the ghost
+    // planes (whole warps of them, for all but the shortest lattices)
+    const bool inside = p.gp[0] < 0 && p.gp[2] < 0;
+    Real js[3];
+    if (inside) set_moments<WITH_P, false>(mc, v, a, p, n, M - 1, sm.rho, js, sm.P);
+    else set_moments<WITH_P, true>(mc, v, a, p, n, M - 1, sm.rho, js, sm.P);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) sm.j[d] = cvt<double>(js[d]);
+    double rest = 0.0;
+#pragma unroll 1
+    for (int s = 0; s < M; ++s) {
+        double ra;
+        Real j[3];
+        if (s < M - 1) {
+            if (inside) set_moments<false, false>(mc, v, a, p, n, s, ra, j, nullptr);
+            else set_moments<false, true>(mc, v, a, p, n, s, ra, j, nullptr);
+            rest += ra;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) js[d] -= j[d];
+        } else {
+            ra = sm.rho - rest;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) j[d] = js[d];
+        }
+        put(s, ra, j);
+    }
+    if (inside)
+        fixed_row_moments<false>([&](auto d) { return pull_g<false>(v, a, decltype(d)::value, p); }, sm.rhoE, sm.q[0],
+                                 sm.q[1], sm.q[2], nullptr);
+    else
+        fixed_row_moments<false>([&](auto d) { return pull_g<true>(v, a, decltype(d)::value, p); }, sm.rhoE, sm.q[0],
+                                 sm.q[1], sm.q[2], nullptr);
 }
 
 // ---------------------------------------------------------------------
@@ -800,14 +856,35 @@ __global__ void __launch_bounds__(LBMK_BLOCK, LBMK_INIT_MINB) k_init(StepArgs a,
 // ---------------------------------------------------------------------
 // Ghost nodes beyond the x faces (Sec. 5a): equilibria at the
 // post-collision moments of the adjacent boundary node, u = 0 on the left.
+//
+// One lane per set: a group of M + 1 lanes forms a ghost node, each lane the
+// sums, then the equilibrium populations, of its set (the energy set's are
+// dealt out over the group).  There are few ghost nodes (32 in a 4 x 4
+// tube), so the kernel's time is the serial chain of one thread, 64 cycles
+// per double operation: 86 us in a 4 x 4 tube with one thread per node, 19
+// (double) and 25 us (mixed) with a group; 34 instead of 125 us for 48 tubes.
 // ---------------------------------------------------------------------
 template <int M>
-__device__ __forceinline__ void ghost_node(const StepArgs &a, int t)
+constexpr int ghost_groups() { return 32 / (M + 1); }      // ghost nodes per warp
+
+__host__ __device__ inline int ghost_count(const StepArgs &a) { return 2 * (a.nseg > 1 ? a.nseg : 1) * a.ny * a.nz; }
+
+// The ghost nodes of warp w (whole warps only).
+template <int M>
+__device__ __forceinline__ void ghost_warp(const StepArgs &a, int w)
 {
+    constexpr int S = M + 1;
     const MechConst &mc = c_mech[a.slot];
-    const int plane = a.ny * a.nz;
-    const int nlat = a.nseg > 1 ? a.nseg : 1;
-    if (t >= 2 * nlat * plane) return;
+    const int lane = threadIdx.x & 31, plane = a.ny * a.nz;
+    int grp = lane / S;
+    const int s = lane % S;
+    int t = w * ghost_groups<M>() + grp;
+    const bool live = grp < ghost_groups<M>() && t < ghost_count(a);
+    if (!live) {                                       // idle lanes follow the first node
+        t = w * ghost_groups<M>();
+        grp = 0;
+    }
+    const int base = grp * S;
     const int gp = t / plane, yz = t % plane;          // ghost plane 2k + side of lattice k
     const int side = gp & 1, k = gp >> 1;
     int x0 = 0, x1 = a.nx;
@@ -819,40 +896,82 @@ __device__ __forceinline__ void ghost_node(const StepArgs &a, int t)
     size_t n = (size_t)(side ? x1 - 1 : x0) + (size_t)a.nx * yz;
     if (!index_ok(x0 >= 0 && x0 < x1 && x1 <= a.nx && n < (size_t)a.N, a.status)) n = 0;
     const PopView v = view(a.src, a);
-    double rho_a[M], rho = 0.0, j[3] = {0, 0, 0}, rhoE = 0.0;
-    double rest = 0.0;
-    for (int s = 0; s < M - 1; ++s) {
-        double acc = 0.0;
-        for (int i = 0; i < LBMK_Q; ++i) acc += load_sf_d(mc, v, s, i, n);
-        rho_a[s] = acc;
-        rest += acc;
-    }
-    for (int i = 0; i < LBMK_Q; ++i) {
-        const double f = load_sf_d(mc, v, M - 1, i, n);
-        rho += f;
-        j[0] += CX(i) * f;
-        j[1] += CY(i) * f;
-        j[2] += CZ(i) * f;
-        rhoE += load_g(v, i, n);
-    }
-    rho_a[M - 1] = rho - rest;
-    double Y[M];
+    double m0, mx, my, mz;
+    row_moments<false, double>([&](auto d) {
+        constexpr int I = decltype(d)::value;
+        return s < M ? load_sf_d(mc, v, s, I, n) : load_g(v, I, n);
+    }, m0, mx, my, mz, nullptr);
+    auto from = [&](double x, int set) { return __shfl_sync(0xffffffffu, x, base + set); };
+    const double rho = from(m0, M - 1), rhoE = from(m0, M), ir = 1.0 / rho;
+    double u[3] = {from(mx, M - 1) * ir, from(my, M - 1) * ir, from(mz, M - 1) * ir};
+    double Y[M], rest = 0.0, inv_m = 0.0;
 #pragma unroll
-    for (int s = 0; s < M; ++s) Y[s] = rho_a[s] / rho;
-    double u[3] = {j[0] / rho, j[1] / rho, j[2] / rho};
-    const double e = rhoE / rho - 0.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    for (int b = 0; b < M - 1; ++b) {
+        const double ra = from(m0, b);
+        rest += ra;
+        Y[b] = ra * ir;
+    }
+    Y[M - 1] = (rho - rest) * ir;
+#pragma unroll
+    for (int b = 0; b < M; ++b) inv_m = fma(Y[b], mc.invW[b], inv_m);
+    // coefficients of the mixture energy, dealt out over the group
     double eu[6];
-    mixture_energy_poly<M>(mc, Y, eu);
+    {
+        constexpr int NK = (6 + S - 1) / S;
+        double part[NK];
+#pragma unroll
+        for (int j = 0; j < NK; ++j) {
+            const int kk = s + j * S < 6 ? s + j * S : 0;
+            part[j] = 0.0;
+#pragma unroll
+            for (int b = 0; b < M; ++b) part[j] = fma(Y[b], mc.uco[b][kk], part[j]);
+        }
+#pragma unroll
+        for (int q = 0; q < 6; ++q) eu[q] = from(part[q / S], q % S);
+    }
+    const double e = rhoE * ir - 0.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
     const double T = solve_T(eu, e, a.macro[(size_t)DR_T * a.N + n], a.status);
     if (side == 0) u[0] = u[1] = u[2] = 0.0;
-    double *gh = static_cast<double *>(a.ghost) + (size_t)gp * (M + 1) * LBMK_Q * plane;
-    equilibria<M>(mc, rho_a, u, T, [&](int s, int i, double val) { gh[((size_t)s * LBMK_Q + i) * plane + yz] = val; });
+    const double Rm = mc.r_lat * inv_m;
+    double *gh = static_cast<double *>(a.ghost) + (size_t)gp * S * LBMK_Q * plane + yz;
+    if (s < M) {
+        const double zeta = (s < M - 1 ? mc.Ra[s] : Rm) * T;
+        const double r = s < M - 1 ? m0 : rho;
+        double P3[3][3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+#pragma unroll
+            for (int c = -1; c <= 1; ++c) P3[d][c + 1] = psi_c(c, u[d], u[d] * u[d] + zeta);
+#pragma unroll
+        for (int cz = 0; cz < 3; ++cz)
+#pragma unroll
+            for (int cy = 0; cy < 3; ++cy) {
+                const double ryz = r * P3[2][cz] * P3[1][cy];
+#pragma unroll
+                for (int cx = 0; cx < 3; ++cx)
+                    if (live) gh[((size_t)s * LBMK_Q + cx + 3 * cy + 9 * cz) * plane] = ryz * P3[0][cx];
+            }
+    }
+    // energy set: rho E and H of the state with the ghost's velocity
+    const double U = poly5(eu, T), usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    const double rE = rho * (U + 0.5 * usq), P = rho * Rm * T;
+    double q[3], Rt[6], tr3;
+    energy_moments(rho, u, P, U + Rm * T + 0.5 * usq, rE, q, Rt, tr3);
+    for (int i = s; i < LBMK_Q; i += S)
+        if (live) gh[((size_t)M * LBMK_Q + i) * plane] = grad_dir(i, rE, q, Rt, tr3);
 }
 
 template <int M>
-__global__ void __launch_bounds__(LBMK_BLOCK) k_ghost(StepArgs a)
+__global__ void __launch_bounds__(32) k_ghost(StepArgs a)
 {
-    ghost_node<M>(a, blockIdx.x * blockDim.x + threadIdx.x);
+    ghost_warp<M>(a, blockIdx.x);
+}
+
+template <int M>
+void launch_ghost(const StepArgs &a)
+{
+    const int nb = (ghost_count(a) + ghost_groups<M>() - 1) / ghost_groups<M>();
+    k_ghost<M><<<nb, 32, 0, a.stream>>>(a);
 }
 
 // ---------------------------------------------------------------------
@@ -1066,6 +1185,31 @@ __device__ __forceinline__ void molar_production(const MechConst &mc, double T, 
     }
 }
 
+// The temperature of a node from its pulled populations, with the moments in
+// sm and the densities rho_a in M columns of shared memory (this thread's,
+// stride bs); eu: the coefficients of the mixture energy, when asked for.
+template <int M>
+__device__ __forceinline__ double node_temperature(const MechConst &mc, const StepArgs &a, const PullIdx &p, int n,
+                                                   Sums &sm, double *sh_ra, int bs, double *eu_out = nullptr)
+{
+    double ir = 0.0, eu[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) eu[k] = 0.0;
+    pull_moments<M, false>(mc, a, p, n, sm, [&](int s, double ra, const Real *) {
+        if (s == 0) ir = 1.0 / sm.rho;
+        const double Y = ra * ir;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) eu[k] = fma(Y, mc.uco[s][k], eu[k]);
+        sh_ra[s * bs] = ra;
+    });
+    const double u[3] = {sm.j[0] * ir, sm.j[1] * ir, sm.j[2] * ir};
+    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    if (eu_out)
+#pragma unroll
+        for (int k = 0; k < 6; ++k) eu_out[k] = eu[k];
+    return solve_T(eu, sm.rhoE * ir - 0.5 * usq, a.macro[(size_t)DR_T * a.N + n], a.status);
+}
+
 // ---------------------------------------------------------------------
 // Moments for lbm_moments: the fields of the state in src (no record).
 // ---------------------------------------------------------------------
@@ -1080,44 +1224,57 @@ __global__ void __launch_bounds__(LBMK_BLOCK, LBMK_MOM_MINB) k_moments(StepArgs 
     if (!node_of(nd, a)) return;
     PullIdx p;
     make_pull(p, nd, a);
-    double rho_a[M];
-    Real ja[M][3];
-    Sums sm;
-    pull_moments<M, false>(mc, a, p, nd.n, rho_a, ja, sm);
-    const double rho = sm.rho;
-    double rest = 0.0;
-#pragma unroll
-    for (int s = 0; s < M - 1; ++s) rest += rho_a[s];
-    rho_a[M - 1] = rho - rest;
-    double Y[M], inv_m = 0.0;
-#pragma unroll
-    for (int s = 0; s < M; ++s) { Y[s] = rho_a[s] / rho; inv_m += Y[s] * mc.invW[s]; }
-    const double u[3] = {sm.j[0] / rho, sm.j[1] / rho, sm.j[2] / rho};
-    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    double eu[6];
-    mixture_energy_poly<M>(mc, Y, eu);
     const int n = nd.n;
     const size_t N = a.N;
-    const double T = solve_T(eu, sm.rhoE / rho - 0.5 * usq, a.macro[DR_T * N + n], a.status);
-    const double Rm = mc.r_lat * inv_m;
+    // rows of out: the fields of the mask in bit order
     size_t row = 0;
-    if (mask & 1u) { for (int s = 0; s < M; ++s) out[(row + s) * N + n] = rho_a[s]; row += M; }
-    if (mask & 2u) { for (int d = 0; d < 3; ++d) out[(row + d) * N + n] = sm.j[d]; row += 3; }
-    if (mask & 4u) { out[row * N + n] = sm.rhoE; row += 1; }
-    if (mask & 8u) { out[row * N + n] = T; row += 1; }
-    if (mask & 16u) { out[row * N + n] = rho * Rm * T; row += 1; }
-    if (mask & 32u) { for (int s = 0; s < M; ++s) out[(row + s) * N + n] = Y[s]; row += M; }
-    if (mask & 64u) {
-        double jM[3] = {sm.j[0], sm.j[1], sm.j[2]};
-        for (int s = 0; s < M - 1; ++s)
-            for (int d = 0; d < 3; ++d) { out[(row + 3 * s + d) * N + n] = ja[s][d]; jM[d] -= ja[s][d]; }
-        for (int d = 0; d < 3; ++d) out[(row + 3 * (M - 1) + d) * N + n] = jM[d];
-        row += 3 * M;
-    }
+    auto rows = [&](unsigned bit, int count) {
+        const size_t r = row;
+        if (mask & bit) row += count;
+        return out + r * N + n;
+    };
+    double *o_ra = rows(1u, M), *o_j = rows(2u, 3), *o_E = rows(4u, 1), *o_T = rows(8u, 1), *o_P = rows(16u, 1),
+           *o_Y = rows(32u, M), *o_ja = rows(64u, 3 * M);
+    Sums sm = {};
+    double ir = 0.0, inv_m = 0.0, eu[6], jM[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) eu[k] = 0.0;
+    pull_moments<M, false>(mc, a, p, n, sm, [&](int s, double ra, const Real *j) {
+        if (s == 0) {
+            ir = 1.0 / sm.rho;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) jM[d] = sm.j[d];
+        }
+        const double Y = ra * ir;
+        inv_m = fma(Y, mc.invW[s], inv_m);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) eu[k] = fma(Y, mc.uco[s][k], eu[k]);
+        sh_act[s * LBMK_BLOCK + threadIdx.x] = ra;
+        if (mask & 1u) o_ra[(size_t)s * N] = ra;
+        if (mask & 32u) o_Y[(size_t)s * N] = Y;
+        if (mask & 64u)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const double jd = s < M - 1 ? cvt<double>(j[d]) : jM[d];
+                o_ja[(size_t)(3 * s + d) * N] = jd;
+                jM[d] -= jd;
+            }
+    });
+    const double rho = sm.rho;
+    const double u[3] = {sm.j[0] * ir, sm.j[1] * ir, sm.j[2] * ir};
+    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    const double T = solve_T(eu, sm.rhoE * ir - 0.5 * usq, a.macro[DR_T * N + n], a.status);
+    const double Rm = mc.r_lat * inv_m;
+    if (mask & 2u)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) o_j[(size_t)d * N] = sm.j[d];
+    if (mask & 4u) *o_E = sm.rhoE;
+    if (mask & 8u) *o_T = T;
+    if (mask & 16u) *o_P = rho * Rm * T;
     if (mask & (128u | 256u)) {
         double conc[M];
 #pragma unroll
-        for (int s = 0; s < M; ++s) conc[s] = rho_a[s] * mc.invW[s];
+        for (int s = 0; s < M; ++s) conc[s] = sh_act[s * LBMK_BLOCK + threadIdx.x] * mc.invW[s];
         molar_production<M>(mc, T, conc, sh_act, sh_g, sh_w, threadIdx.x, LBMK_BLOCK);
         if (mask & 128u) {
             for (int s = 0; s < M; ++s) out[(row + s) * N + n] = mc.W[s] * (double)sh_w[s * LBMK_BLOCK + threadIdx.x];
@@ -1161,84 +1318,23 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd, doub
     const size_t N = a.N;
     const RecRows rr = rec_rows(M, LBMK_MIXED);
     Real *R = rec(a);
-    const PopView v = view(a.src, a);
     PullIdx p;
     make_pull(p, nd, a);
-    // population of set s, direction I; in the mixed units its deviation
-    // from the rest state (the double rest populations are added below)
-    auto pull = [&](int s, auto d) {
-        constexpr int I = decltype(d)::value;
-#if LBMK_MIXED
-        if (I == REST) return (Real)0;
-        return pull_dev(mc, v, a, s, I, p);
-#else
-        return pull_sf(mc, v, a, s, I, p);
-#endif
-    };
-    auto rest_part = [&](int s) {
-#if LBMK_MIXED
-        return mc.ref0[s] + v.rest()[(size_t)s * N + n];
-#else
-        (void)s;
-        return 0.0;
-#endif
-    };
-
-    // mixture set
-    double rho, P2[6];
-    Real js[3];
-    {
-        Real a0, P6[6];
-        row_moments<true, Real>([&](auto d) { return pull(M - 1, d); }, a0, js[0], js[1], js[2], P6);
-        rho = cvt<double>(a0);
-#if LBMK_MIXED
-        rho += rest_part(M - 1);
-#endif
-#pragma unroll
-        for (int k = 0; k < 6; ++k) P2[k] = cvt<double>(P6[k]);
-#if LBMK_MIXED
-#pragma unroll
-        for (int d = 0; d < 3; ++d) P2[d] += mc.refP[M - 1][d];
-#endif
-    }
-    const double ir = 1.0 / rho;
-    const double u[3] = {cvt<double>(js[0]) * ir, cvt<double>(js[1]) * ir, cvt<double>(js[2]) * ir};
-    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-
-    // species densities and momenta; the last species is slaved (Eq. (strongest))
-    double rest = 0.0, inv_m = 0.0, eu[6];
+    Sums sm = {};
+    double ir = 0.0, inv_m = 0.0, eu[6];
     bool neg = false;
 #pragma unroll
     for (int k = 0; k < 6; ++k) eu[k] = 0.0;
-#pragma unroll 1
-    for (int s = 0; s < M; ++s) {
-        double ra;
-        Real jx, jy, jz;
-        if (s < M - 1) {
-            Real a0;
-            row_moments<false, Real>([&](auto d) { return pull(s, d); }, a0, jx, jy, jz, nullptr);
-            ra = cvt<double>(a0);
-#if LBMK_MIXED
-            ra += rest_part(s);
-#endif
-            rest += ra;
-            js[0] -= jx;
-            js[1] -= jy;
-            js[2] -= jz;
-        } else {
-            ra = rho - rest;
-            jx = js[0];
-            jy = js[1];
-            jz = js[2];
-        }
+    pull_moments<M, true>(mc, a, p, n, sm, [&](int s, double ra, const Real *j) {
+        if (s == 0) ir = 1.0 / sm.rho;
         Real *J = R + (size_t)(rr.du + 3 * s) * N + n;
-        J[0] = jx;
-        J[N] = jy;
-        J[2 * N] = jz;
+        J[0] = j[0];
+        J[N] = j[1];
+        J[2 * N] = j[2];
         const double Y = ra * ir;
         inv_m = fma(Y, mc.invW[s], inv_m);
         if (__double2hiint(ra) < 0)             // sign bit first: the compare only for negative values
-            neg |= ra < -1e-10 * rho;           // below rounding noise of trace species
+            neg |= ra < -1e-10 * sm.rho;        // below rounding noise of trace species
 #pragma unroll
         for (int k = 0; k < 6; ++k) eu[k] = fma(Y, mc.uco[s][k], eu[k]);
         sh[s * bs] = ra;
@@ -1249,12 +1345,10 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd, doub
 #else
         R[(size_t)(rr.ra + s) * N + n] = ra;
 #endif
-    }
-
-    // energy set
-    double rhoE, q[3];
-    row_moments<false, double>([&](auto d) { return pull_g(v, a, decltype(d)::value, p); }, rhoE, q[0], q[1], q[2],
-                               nullptr);
+    });
+    const double rho = sm.rho, rhoE = sm.rhoE;
+    const double u[3] = {sm.j[0] * ir, sm.j[1] * ir, sm.j[2] * ir};
+    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
     if (!(rho > 0.0) || !isfinite(rhoE)) flag(a.status, LBMK_BIT_NONFINITE);
     if (neg) flag(a.status, LBMK_BIT_NEGATIVE);
 
@@ -1303,9 +1397,9 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd, doub
     // (Eq. (corrFourier)) needs the neighbours and is added in k_step_g.
     double qeq[3], Rt[6], tr3;
     energy_moments(rho, u, P, H + 0.5 * usq, rhoE, qeq, Rt, tr3);
-    const double dP[6] = {P2[0] - (P + rho * u[0] * u[0]), P2[1] - (P + rho * u[1] * u[1]),
-                          P2[2] - (P + rho * u[2] * u[2]), P2[3] - rho * u[0] * u[1],
-                          P2[4] - rho * u[0] * u[2], P2[5] - rho * u[1] * u[2]};
+    const double dP[6] = {sm.P[0] - (P + rho * u[0] * u[0]), sm.P[1] - (P + rho * u[1] * u[1]),
+                          sm.P[2] - (P + rho * u[2] * u[2]), sm.P[3] - rho * u[0] * u[1],
+                          sm.P[4] - rho * u[0] * u[2], sm.P[5] - rho * u[1] * u[2]};
     const double uP[3] = {u[0] * dP[0] + u[1] * dP[3] + u[2] * dP[4], u[0] * dP[3] + u[1] * dP[1] + u[2] * dP[5],
                           u[0] * dP[4] + u[1] * dP[5] + u[2] * dP[2]};
 
@@ -1332,7 +1426,7 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd, doub
         R[(size_t)(rr.phi + d) * N + n] = rhoR * ud * (ph - ud * ud);
         R[(size_t)(rr.u + d) * N + n] = ud;
         // the difference is formed in double (it cancels), the product in the storage type
-        R[(size_t)(rr.dq + d) * N + n] = (omega - omega1) * cvt<Real>(q[d] - uP[d] - qeq[d]);
+        R[(size_t)(rr.dq + d) * N + n] = (omega - omega1) * cvt<Real>(sm.q[d] - uP[d] - qeq[d]);
     }
     R[(size_t)rr.rho * N + n] = rhoR;
     R[(size_t)rr.kappa * N + n] = cvt<Real>(kappa);
@@ -1918,10 +2012,7 @@ int launch_one(const StepArgs &a, int k)
     const int bs = a.bs[k];
     switch (k) {
     case LBMK_K_GHOST:
-        if (a.bc_x == 1) {
-            const int plane = a.ny * a.nz;
-            k_ghost<M><<<grid_for(2 * (a.nseg > 1 ? a.nseg : 1) * plane), LBMK_BLOCK, 0, a.stream>>>(a);
-        }
+        if (a.bc_x == 1) launch_ghost<M>(a);
         break;
     case LBMK_K_PRE: {
         k_pre<M><<<grid_for(a.N, bs), bs, pre_cols<M>() * bs * sizeof(double), a.stream>>>(a);
@@ -2019,8 +2110,9 @@ template <int M, bool FX>
 __device__ __forceinline__ bool persist_step(const StepArgs &b, int tile, GridBarrier *bar, unsigned nb, unsigned cap)
 {
     if (b.bc_x == 1) {
-        const int ng = 2 * (b.nseg > 1 ? b.nseg : 1) * b.ny * b.nz;
-        for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x) ghost_node<M>(b, g);
+        const int nw = (ghost_count(b) + ghost_groups<M>() - 1) / ghost_groups<M>();
+        const int per = blockDim.x / 32;
+        for (int w = blockIdx.x + gridDim.x * (threadIdx.x / 32); w < nw; w += gridDim.x * per) ghost_warp<M>(b, w);
         if (!grid_barrier(bar, nb, cap, b.status)) return false;
     }
     tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) {
@@ -2104,10 +2196,7 @@ int run_step(const StepArgs &a, cudaEvent_t *ev)
 template <int M>
 int run_moments(const StepArgs &a, unsigned mask, double *out)
 {
-    if (a.bc_x == 1) {
-        const int plane = a.ny * a.nz;
-        k_ghost<M><<<grid_for(2 * (a.nseg > 1 ? a.nseg : 1) * plane), LBMK_BLOCK, 0, a.stream>>>(a);
-    }
+    if (a.bc_x == 1) launch_ghost<M>(a);
     k_moments<M><<<grid_for(a.N), LBMK_BLOCK, 0, a.stream>>>(a, mask, out);
     return (int)cudaGetLastError();
 }
@@ -2357,6 +2446,7 @@ __global__ void __launch_bounds__(LBMK_HRR_THREADS, 3) k_hrr(StepArgs a, double 
 {
     __shared__ double sh_dA[LBMK_MAXR * LBMK_HRR_THREADS];
     __shared__ double sh_J[LBMK_HRR_THREADS];
+    __shared__ double sh_ra[M * LBMK_HRR_THREADS];
     const MechConst &mc = c_mech[a.slot];
     const int t = threadIdx.x, R = mc.R;
     const size_t N = a.N;
@@ -2368,24 +2458,11 @@ __global__ void __launch_bounds__(LBMK_HRR_THREADS, 3) k_hrr(StepArgs a, double 
         node_at(nd, a);
         PullIdx p;
         make_pull(p, nd, a);
+        Sums sm = {};
+        const double T = node_temperature<M>(mc, a, p, n, sm, sh_ra + t, LBMK_HRR_THREADS);
         double rho_a[M];
-        Real ja[M][3];
-        Sums sm;
-        pull_moments<M, false>(mc, a, p, n, rho_a, ja, sm);
-        // the node state as in k_moments
-        const double rho = sm.rho;
-        double rest = 0.0;
 #pragma unroll
-        for (int s = 0; s < M - 1; ++s) rest += rho_a[s];
-        rho_a[M - 1] = rho - rest;
-        double Y[M];
-#pragma unroll
-        for (int s = 0; s < M; ++s) Y[s] = rho_a[s] / rho;
-        const double u[3] = {sm.j[0] / rho, sm.j[1] / rho, sm.j[2] / rho};
-        const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-        double eu[6];
-        mixture_energy_poly<M>(mc, Y, eu);
-        const double T = solve_T(eu, sm.rhoE / rho - 0.5 * usq, a.macro[DR_T * N + n], a.status);
+        for (int s = 0; s < M; ++s) rho_a[s] = sh_ra[s * LBMK_HRR_THREADS + t];
         double dT, drho[M];
         Jt += hrr_node<M>(mc, T, rho_a, &dT, drho, sh_dA + t, LBMK_HRR_THREADS);
         if (dT_out) dT_out[n] = dT;
@@ -2488,10 +2565,7 @@ __global__ void __launch_bounds__(LBMK_HRR_THREADS) k_hrr_final(const double *pa
 template <int M>
 int run_hrr(const StepArgs &a, int R, double *dT, double *drho, double *partial, double *out)
 {
-    if (a.bc_x == 1) {
-        const int plane = a.ny * a.nz;
-        k_ghost<M><<<grid_for(2 * (a.nseg > 1 ? a.nseg : 1) * plane), LBMK_BLOCK, 0, a.stream>>>(a);
-    }
+    if (a.bc_x == 1) launch_ghost<M>(a);
     const int nb = lbmk::hrr_blocks(a.N);
     k_hrr<M><<<nb, LBMK_HRR_THREADS, 0, a.stream>>>(a, dT, drho, partial);
     k_hrr_final<<<1 + R, LBMK_HRR_THREADS, 0, a.stream>>>(partial, nb, 1 + R, out);
@@ -2545,23 +2619,18 @@ __global__ void __launch_bounds__(LBMK_HRR_THREADS, 3) k_hrr_adj(StepArgs a, dou
     node_at(nd, a);
     PullIdx p;
     make_pull(p, nd, a);
-    double rho_a[M];
-    Real ja[M][3];
+    __shared__ double sh_ra[M * LBMK_HRR_THREADS];
     Sums sm;
-    pull_moments<M, false>(mc, a, p, n, rho_a, ja, sm);
-    const double rho = sm.rho;
-    double rest = 0.0;
-#pragma unroll
-    for (int s = 0; s < M - 1; ++s) rest += rho_a[s];
-    rho_a[M - 1] = rho - rest;
-    double Y[M];
-#pragma unroll
-    for (int s = 0; s < M; ++s) Y[s] = rho_a[s] / rho;
-    const double u[3] = {sm.j[0] / rho, sm.j[1] / rho, sm.j[2] / rho};
-    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
     double eu[6];
-    mixture_energy_poly<M>(mc, Y, eu);
-    const double T = solve_T(eu, sm.rhoE / rho - 0.5 * usq, a.macro[DR_T * N + n], a.status);
+    const double T = node_temperature<M>(mc, a, p, n, sm, sh_ra + threadIdx.x, LBMK_HRR_THREADS, eu);
+    const double rho = sm.rho;
+    double rho_a[M], Y[M];
+#pragma unroll
+    for (int s = 0; s < M; ++s) {
+        rho_a[s] = sh_ra[s * LBMK_HRR_THREADS + threadIdx.x];
+        Y[s] = rho_a[s] / rho;
+    }
+    const double u[3] = {sm.j[0] / rho, sm.j[1] / rho, sm.j[2] / rho};
     double GT, G[M];
     hrr_node<M, false>(mc, T, rho_a, &GT, G, nullptr, 0);
     const double l = GT / dpoly5(eu, T), ir = 1.0 / rho;
