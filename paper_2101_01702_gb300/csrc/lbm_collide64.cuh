@@ -1,43 +1,51 @@
 // Collisions of the species and mixture sets in double precision (pass 3b
 // of lbm_kernels.cuh, which includes this file in the double units).
 //
-// The kernel is bound by the FP64 pipe.  Per node, direction and species it
-// spends five FP64 operations:
-//   E_b = R_b psi_x(u) psi_y(u) psi_z(u)      (one product; the y-z part of
-//   D_b = E_b - R_b psi_x psi_y psi_z(u+du_b)  a row and the x factors are
-//                                              kept per species)
-//   f_a <- (1 - 2 beta_a) f_a + c_a E_a + g_a sum_b K_ab D_b,
-// R_b = rho Y_b / W_b, c_a = (2 beta_a rho_a + rho_dot_a) / R_a,
-// g_a = (beta_a - 1) kappa Y_a / W_a and K_ab = 1/D_ab, which is Eq.
-// (finalNumericalEquations) with Eq. (fStar) and the factors that do not
-// depend on the direction taken out of it.  The sum over the partner species
-// b -- (M-1)^2 terms per direction, three quarters of what remains at
-// nine species -- runs on the integer pipe (lbm_fixed.cuh): the D_b of a
-// direction are brought to the largest one's exponent, and K to that of
-// its largest entry.
+// The kernel is bound by the FP64 pipe.  With
+//   e_b = psi_x psi_y psi_z at u,  s_b the same at u + du_b (Eq. (phis)),
+//   D_b = R_b (e_b - s_b),  R_b = rho Y_b / W_b,  K_ab = 1/D_ab,
+//   f_a <- (1 - 2 beta_a) f_a + (2 beta_a rho_a + rho_dot_a) e_a
+//          + (beta_a - 1) kappa Y_a / W_a sum_b K_ab D_b,
+// which is Eq. (finalNumericalEquations) with Eq. (fStar) and the factors that
+// do not depend on the direction taken out of it, three FP64 operations
+// per direction and species remain (the product e_a from the y-z part of
+// its row, two multiply-adds).  The differences D_b and the sums over the
+// partner species -- (M-1)^2 terms per direction -- run on the integer pipe
+// (lbm_fixed.cuh): the y-z parts of a row and the x factors of a direction as
+// limbs, each block brought to its largest exponent, and K to that of its
+// largest entry.
 //
 // Measured, 128^3 with nine species, rates included: 33.2 ms with every
-// term formed per direction in floating point, 15.4 ms so (3115 FP64
-// instructions per warp, 86 % of the rate a plain chain of multiply-adds
-// reaches); 1024 nodes with three species: 101 -> 53 us.
+// term formed per direction in floating point; 15.4 ms with the D_b in double
+// and only the sums over b in integers (14.1 ms after the exponentials left
+// the FP64 pipe); 1024 nodes with three species: 101 -> 53 us.
 #pragma once
 
 #include "lbm_fixed.cuh"
 
 namespace {
 
-// Doubles of shared memory per thread: the y and x factors of E and of the
-// quasi-equilibrium for c = -1, 0, 1 (12 per species); before the
-// collision the same columns are the scratch of the production rates.
+// Columns of shared memory per thread: the y factors of e and s and the x
+// factors of e as doubles, the x factors of s as limbs (FX) or doubles, for
+// c = -1, 0, 1 (12 per species); before the collision the same columns are
+// the scratch of the production rates.
 template <int M>
 constexpr int step_cols() { return 12 * M; }
 
-// Whether the cross terms use fixed point: below four species there are at
-// most four products per direction, fewer than the conversions cost.
-template <int M>
-constexpr bool kMixFixed = M >= 4;
+// psi_c(v, v^2 + z) = A + B z with the coefficients of an axis and c.
+struct PsiCoef {
+    double A, B;
+};
+__device__ __forceinline__ PsiCoef psi_coef(int c, double v)
+{
+    const double vsq = v * v;
+    return PsiCoef{c == 0 ? 1.0 - vsq : 0.5 * (c > 0 ? vsq + v : vsq - v), c == 0 ? -1.0 : 0.5};
+}
 
-template <int M>
+// FX: the tables are in the range of the fixed-point sums (MechConst::
+// mix_fixed; from four species on, below there are at most four products
+// per direction, fewer than the conversions cost).
+template <int M, bool FX>
 __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, double *sh, int bs)
 {
     const MechConst &mc = c_mech[a.slot];
@@ -48,8 +56,7 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
     auto ld = [&](int row) { return R[(size_t)row * N + n]; };
 
     const double rho = ld(rr.rho), T = a.macro[(size_t)DR_T * N + n];
-    const bool fixed = kMixFixed<M> && mc.mix_fixed;
-    // per species: R_b, and the factors of f_a, E_a and the cross term
+    // per species: R_b, and the factors of f_a, R_a e_a and the cross term
     double Rw[M], kf[M - 1], kE[M - 1], kF[M - 1];
     {
         double conc[M];
@@ -62,11 +69,11 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
         const double kappa = ld(rr.kappa);
 #pragma unroll
         for (int s = 0; s < M; ++s) {
-            const double wscale = fixed ? mc.invW[s] : 1.0;
+            const double wscale = FX ? mc.invW[s] : 1.0;
             const double ra = Rw[s];
-            // E is scaled by R_b; a species that is absent keeps a scale far
+            // e is scaled by R_b; a species that is absent keeps a scale far
             // below every population, so that its source term survives
-            double r = ra * wscale;
+            double r = FX ? conc[s] : ra;
             r = fabs(r) < 1e-150 ? (r < 0.0 ? -1e-150 : 1e-150) : r;
             Rw[s] = r;
             if (s < M - 1) {
@@ -78,29 +85,45 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
         }
     }
     const double u[3] = {ld(rr.u), ld(rr.u + 1), ld(rr.u + 2)};
-    // psi_c(u, u^2 + z) = eA + eB z per axis and c
-    auto e_factor = [&](int d, int c, double z) {
-        const double usq = u[d] * u[d];
-        return c == 0 ? (1.0 - usq) - z : fma(0.5, z, 0.5 * (usq + (double)c * u[d]));
-    };
-    auto s_factor = [&](int c, double x, double z) {
-        const double sq = fma(x, x, z);
-        return c == 0 ? 1.0 - sq : 0.5 * (sq + (double)c * x);
-    };
+    const double om = ld(rr.om), omf = 1.0 - om, omr = om * rho, RT = ld(rr.rt);
+    int ex[3] = {0, 0, 0};                                  // exponents of the x factors, per c
+    double fx[3];                                           // x factors of the mixture set
+    {
+        PsiCoef q[2][3];
 #pragma unroll
-    for (int s = 0; s < M; ++s) {
-        const double z = mc.Ra[s] * T;
-        double *col = sh + (size_t)(12 * s) * bs + t;
+        for (int c = 0; c < 3; ++c) {
+            q[0][c] = psi_coef(c - 1, u[1]);
+            q[1][c] = psi_coef(c - 1, u[0]);
+            fx[c] = fma(q[1][c].B, RT, q[1][c].A);
+        }
 #pragma unroll
-        for (int d = 0; d < 2; ++d) {                          // d = 0: y factors, d = 1: x factors
-            const int ax = 1 - d;
-            const double x = u[ax] + ld(rr.du + 3 * s + ax);
-            const double sq = fma(x, x, z), hs = 0.5 * sq;
+        for (int s = 0; s < M; ++s) {
+            const double z = mc.Ra[s] * T;
+            double *col = sh + (size_t)(12 * s) * bs + t;
 #pragma unroll
-            for (int c = -1; c <= 1; ++c) {
-                col[(6 * d + c + 1) * bs] = e_factor(ax, c, z);
-                col[(6 * d + 3 + c + 1) * bs] = c == 0 ? 1.0 - sq : fma(0.5 * c, x, hs);
+            for (int d = 0; d < 2; ++d) {                      // d = 0: y factors, d = 1: x factors
+                const int ax = 1 - d;
+                const double x = u[ax] + ld(rr.du + 3 * s + ax);
+                const double sq = fma(x, x, z), hs = 0.5 * sq;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const double e = fma(q[d][c].B, z, q[d][c].A);
+                    const double g = c == 1 ? 1.0 - sq : fma(0.5 * (c - 1), x, hs);
+                    col[(6 * d + c) * bs] = e;
+                    col[(6 * d + 3 + c) * bs] = g;
+                    if (d == 1) ex[c] = max(ex[c], max(biased_exponent(e), biased_exponent(g)));
+                }
             }
+        }
+        if constexpr (FX) {
+#pragma unroll
+            for (int s = 0; s < M; ++s)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    double *x = sh + (size_t)(12 * s + 9 + c) * bs + t;
+                    const Limbs58 v = to_limbs58(*x, ex[c]);
+                    *x = __hiloint2double(v.h, v.l);
+                }
         }
     }
 
@@ -122,81 +145,116 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
 #pragma unroll
         for (int k = 0; k < 3; ++k) X[k] *= -1.5;              // A_i . X = c_i . X / 2 on the axes
     }
-    const double om = ld(rr.om), omf = 1.0 - om, omr = om * rho, RT = ld(rr.rt);
 
     const PopView v = view(a.src, a);
     PullIdx p;
     make_pull(p, nd, a);
+    const size_t set = (size_t)LBMK_Q * N;
     int bad = 0;                                               // a non-finite result (exponent bits)
 #pragma unroll 1
     for (int cz = -1; cz <= 1; ++cz) {
         double zE[M], zS[M];
+        const PsiCoef qz = psi_coef(cz, u[2]);
+        const double sA = cz == 0 ? 1.0 : 0.0, sC = cz == 0 ? 0.0 : (cz > 0 ? 0.5 : -0.5);
 #pragma unroll
         for (int s = 0; s < M; ++s) {
             const double z = mc.Ra[s] * T;
-            zE[s] = Rw[s] * e_factor(2, cz, z);
-            zS[s] = Rw[s] * s_factor(cz, u[2] + ld(rr.du + 3 * s + 2), z);
+            zE[s] = Rw[s] * fma(qz.B, z, qz.A);
+            const double x = u[2] + ld(rr.du + 3 * s + 2);
+            zS[s] = Rw[s] * fma(sC, x, fma(qz.B, fma(x, x, z), sA));
         }
-        const double fz = omr * e_factor(2, cz, RT);
+        const double fz = omr * fma(qz.B, RT, qz.A);
 #pragma unroll 1
         for (int cy = -1; cy <= 1; ++cy) {
-            double pe[M], ps[M];
+            double pe[M], ps[M];                               // R_b psi_y psi_z of e and s
+            int er = 0;
 #pragma unroll
             for (int s = 0; s < M; ++s) {
                 pe[s] = zE[s] * sh[(12 * s + cy + 1) * bs + t];
                 ps[s] = zS[s] * sh[(12 * s + 3 + cy + 1) * bs + t];
+                er = max(er, max(biased_exponent(pe[s]), biased_exponent(ps[s])));
             }
-            const double fyz = fz * e_factor(1, cy, RT);
+            Limbs58 le[M], ls[M];
+            if constexpr (FX) {
+#pragma unroll
+                for (int s = 0; s < M; ++s) {
+                    le[s] = to_limbs58(pe[s], er);
+                    const Limbs58 x = to_limbs58(ps[s], er);
+                    ls[s] = Limbs58{-x.h, -x.l};
+                    if (s < M - 1) pe[s] *= kE[s];
+                }
+            }
+            const PsiCoef qy = psi_coef(cy, u[1]);
+            const double fyz = fz * fma(qy.B, RT, qy.A);
 #pragma unroll 1
             for (int cx = -1; cx <= 1; ++cx) {
                 const int i = (cx + 1) + 3 * (cy + 1) + 9 * (cz + 1);
                 double f[M];
                 const Src sr = src_of(i, p, a);
+                if (sr.ghost) {
 #pragma unroll
-                for (int s = 0; s < M; ++s)
-                    f[s] = sr.ghost ? load_ghost(a, sr.side, s, i, sr.idx) : load_raw_sf(v, s, i, sr.idx);
-                double E[M], D[M];
+                    for (int s = 0; s < M; ++s) f[s] = load_ghost(a, sr.side, s, i, sr.idx);
+                } else {
+                    const double *src = static_cast<const double *>(v.buf) + (size_t)i * N + sr.idx;
 #pragma unroll
-                for (int s = 0; s < M; ++s) {
-                    E[s] = pe[s] * sh[(12 * s + 6 + cx + 1) * bs + t];
-                    D[s] = fma(-ps[s], sh[(12 * s + 9 + cx + 1) * bs + t], E[s]);
+                    for (int s = 0; s < M; ++s) f[s] = LBMK_LDG(src + s * set);
                 }
-                double F[M - 1];
-                if (fixed) {
-                    int e = 0;
+                double E[M], F[M - 1];
+                if constexpr (FX) {
+                    const int exc = cx < 0 ? ex[0] : (cx == 0 ? ex[1] : ex[2]);
+                    Limbs58 D[M];
 #pragma unroll
-                    for (int b = 0; b < M; ++b) e = max(e, biased_exponent(D[b]));
-                    Limbs58 x[M];
-#pragma unroll
-                    for (int b = 0; b < M; ++b) x[b] = to_limbs58(D[b], e);
+                    for (int s = 0; s < M; ++s) {
+                        const double xe = sh[(12 * s + 6 + cx + 1) * bs + t], xs = sh[(12 * s + 9 + cx + 1) * bs + t];
+                        E[s] = pe[s] * xe;                     // (2 beta_a rho_a + rho_dot_a) e_a; not used for the last
+                        const Limbs58 l = to_limbs58(xe, exc), m{__double2hiint(xs), __double2loint(xs)};
+                        long long hi = 0, mid = 0;
+                        fma_limbs58(hi, mid, le[s].h, le[s].l, l);
+                        fma_limbs58(hi, mid, ls[s].h, ls[s].l, m);
+                        const long long d = hi + (mid >> 29);  // below 2^59
+                        D[s] = Limbs58{(int)(d >> 29), (int)((unsigned)d & 0x1fffffffu)};
+                    }
+                    const int e = er + exc - 2044 + mc.mix_exp;
+                    const bool nan = er == 0x7ff || exc == 0x7ff;      // an infinite or NaN factor
 #pragma unroll
                     for (int s = 0; s < M - 1; ++s) {
                         long long hi = 0, mid = 0;
 #pragma unroll
                         for (int b = 0; b < M; ++b)
-                            if (b != s) fma_limbs58(hi, mid, mc.mixh[s][b], mc.mixl[s][b], x[b]);
-                        F[s] = double_of_int64(hi + (mid >> 29), e - 1022 + mc.mix_exp);
-                        if (e == 0x7ff) F[s] = __longlong_as_double(0x7ff8000000000000ll);   // as D is
+                            if (b != s) fma_limbs58(hi, mid, mc.mixh[s][b], mc.mixl[s][b], D[b]);
+                        F[s] = double_of_int64(hi + (mid >> 29), e);
+                        if (nan) F[s] = __longlong_as_double(0x7ff8000000000000ll);
                     }
                 } else {
+                    double D[M];
+#pragma unroll
+                    for (int s = 0; s < M; ++s) {
+                        E[s] = pe[s] * sh[(12 * s + 6 + cx + 1) * bs + t];
+                        D[s] = fma(-ps[s], sh[(12 * s + 9 + cx + 1) * bs + t], E[s]);
+                    }
 #pragma unroll
                     for (int s = 0; s < M - 1; ++s) {
                         F[s] = 0.0;
 #pragma unroll
                         for (int b = 0; b < M; ++b)
                             if (b != s) F[s] = fma(mc.inv_WWD[s][b], D[b], F[s]);
+                        E[s] *= kE[s];
                     }
                 }
+                double *dst = static_cast<double *>(a.dst) + (size_t)i * N + n;
 #pragma unroll
                 for (int s = 0; s < M - 1; ++s) {
-                    const double val = fma(kf[s], f[s], fma(kE[s], E[s], kF[s] * F[s]));
-                    store_raw(a.dst, a, s, i, n, val);
+                    const double val = fma(kf[s], f[s], fma(kF[s], F[s], E[s]));
+                    dst[s * set] = val;
                     bad |= !finite_bits(val);
                 }
                 // mixture f: Eq. (f) with the isotropy correction A_i . X (Eq. (Ai))
-                double val = fma(omf, f[M - 1], fyz * e_factor(0, cx, RT));
-                if ((cx != 0) + (cy != 0) + (cz != 0) == 1) val += cx * X[0] + cy * X[1] + cz * X[2];
-                store_raw(a.dst, a, M - 1, i, n, val);
+                double val = fma(omf, f[M - 1], fyz * (cx < 0 ? fx[0] : (cx == 0 ? fx[1] : fx[2])));
+                if ((cx != 0) + (cy != 0) + (cz != 0) == 1) {
+                    const double ax = cx ? X[0] : (cy ? X[1] : X[2]);
+                    val += cx + cy + cz < 0 ? -ax : ax;
+                }
+                dst[(M - 1) * set] = val;
                 bad |= !finite_bits(val);
             }
         }

@@ -88,6 +88,11 @@ typedef double WReal;
 #ifndef LBMK_DIFF_MINB
 #define LBMK_DIFF_MINB (LBMK_FAST ? 5 : 2)
 #endif
+// The persistent kernel takes the budget of its heaviest phase, the species
+// collision (the double one's shared memory allows two blocks).
+#ifndef LBMK_PERSIST_MINB
+#define LBMK_PERSIST_MINB (LBMK_MIXED ? 3 : 2)
+#endif
 #ifndef LBMK_STEP_MINB
 #define LBMK_STEP_MINB (LBMK_MIXED ? 3 : 1)
 #endif
@@ -1777,7 +1782,7 @@ __global__ void __launch_bounds__(LBMK_MAXBLOCK) k_step_g(StepArgs a)
 template <int M>
 constexpr int step_cols() { return 3 * M; }      // scratch columns of the production rates
 
-template <int M>
+template <int M, bool FX>
 __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, double *sh, int bs)
 {
     double *sh_act = sh, *sh_g = sh + M * bs;
@@ -1969,18 +1974,23 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
 namespace {
 #endif
 
+// Whether the collision has a variant with fixed-point sums: the double one,
+// from four species on.
+template <int M>
+constexpr bool kFixedStep = M >= 4 && !LBMK_MIXED;
+
 // Shared memory of a block of bs threads for step_node.
 template <int M>
 constexpr size_t step_smem(int bs) { return (size_t)step_cols<M>() * bs * sizeof(double); }
 
 extern __shared__ double sh_step[];
 
-template <int M>
+template <int M, bool FX>
 __global__ void __launch_bounds__(LBMK_BLOCK, LBMK_STEP_MINB) k_step(StepArgs a)
 {
     Node nd;
     if (!node_of(nd, a)) return;
-    step_node<M>(a, nd, sh_step, blockDim.x);
+    step_node<M, FX>(a, nd, sh_step, blockDim.x);
 }
 
 // Opts kernel f in to dynamic shared memory above 48 KB, once per device
@@ -2003,6 +2013,16 @@ int opt_in_smem(F *f, size_t bytes, std::atomic<unsigned long long> &done)
 // Host launchers
 // ---------------------------------------------------------------------
 inline dim3 grid_for(int n, int bs = LBMK_BLOCK) { return dim3((unsigned)((n + bs - 1) / bs)); }
+
+template <int M, bool FX>
+int launch_step(const StepArgs &a, int bs)
+{
+    static std::atomic<unsigned long long> opted{0};
+    const int e = opt_in_smem(k_step<M, FX>, step_smem<M>(LBMK_BLOCK), opted);
+    if (e) return e;
+    k_step<M, FX><<<grid_for(a.N, bs), bs, step_smem<M>(bs), a.stream>>>(a);
+    return 0;
+}
 
 // Launch of one kernel of the step with the context's block size for it
 // (LBMK_K_*; the autotuner times them one at a time).
@@ -2027,10 +2047,9 @@ int launch_one(const StepArgs &a, int k)
     case LBMK_K_GRAD: k_grad<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
     case LBMK_K_STEPG: k_step_g<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
     case LBMK_K_STEP: {
-        static std::atomic<unsigned long long> opted{0};
-        const int e = opt_in_smem(k_step<M>, step_smem<M>(LBMK_BLOCK), opted);
+        constexpr bool FX = kFixedStep<M>;
+        const int e = FX && a.fixed ? launch_step<M, FX>(a, bs) : launch_step<M, false>(a, bs);
         if (e) return e;
-        k_step<M><<<grid_for(a.N, bs), bs, step_smem<M>(bs), a.stream>>>(a);
         break;
     }
     default: return (int)cudaErrorInvalidValue;
@@ -2117,7 +2136,7 @@ __device__ __forceinline__ bool persist_step(const StepArgs &b, int tile, GridBa
     }
     tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) {
         pre_node<M>(b, nd, sh_step + threadIdx.x, LBMK_BLOCK);
-        diff_node<M, FX>(b, nd, sh_step + threadIdx.x, LBMK_BLOCK);
+        diff_node<M, FX && kRefined<M, true>>(b, nd, sh_step + threadIdx.x, LBMK_BLOCK);
     });
     if (!grid_barrier(bar, nb, cap, b.status)) return false;
     tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) { grad_node<M>(b, nd); });
@@ -2127,7 +2146,7 @@ __device__ __forceinline__ bool persist_step(const StepArgs &b, int tile, GridBa
     // each one's arithmetic as in its own kernel (no values shared)
     tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) { collide_energy<M>(b, nd); });
     if (!grid_barrier(bar, nb, cap, b.status)) return false;
-    tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) { step_node<M>(b, nd, sh_step, LBMK_BLOCK); });
+    tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) { step_node<M, FX && kFixedStep<M>>(b, nd, sh_step, LBMK_BLOCK); });
     return grid_barrier(bar, nb, cap, b.status);
 }
 
@@ -2135,7 +2154,7 @@ __device__ __forceinline__ bool persist_step(const StepArgs &b, int tile, GridBa
 // alternate between the two parameter blocks, which the phases then read
 // in place (no per-step copy of the arguments)
 template <int M, bool FX>
-__global__ void __launch_bounds__(LBMK_BLOCK, LBMK_PRE_MINB) k_persist(StepArgs a0, StepArgs a1, int nsteps, int tile,
+__global__ void __launch_bounds__(LBMK_BLOCK, LBMK_PERSIST_MINB) k_persist(StepArgs a0, StepArgs a1, int nsteps, int tile,
                                                                       GridBarrier *bar, unsigned cap)
 {
     const unsigned nb = gridDim.x;
@@ -2175,8 +2194,8 @@ int launch_persistent(const StepArgs &a, int nsteps, int tile_mult, GridBarrier 
 template <int M>
 int run_persistent(const StepArgs &a, int nsteps, int tile_mult, GridBarrier *bar, unsigned cap)
 {
-    if (kRefined<M, true> && a.fixed)
-        return launch_persistent<M, kRefined<M, true>>(a, nsteps, tile_mult, bar, cap);
+    constexpr bool FX = kRefined<M, true> || kFixedStep<M>;
+    if (FX && a.fixed) return launch_persistent<M, FX>(a, nsteps, tile_mult, bar, cap);
     return launch_persistent<M, false>(a, nsteps, tile_mult, bar, cap);
 }
 #endif  // LBMK_COHERENT_LOADS
