@@ -180,7 +180,7 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
                 for (int s = 0; s < M; ++s) {
                     le[s] = to_limbs58(pe[s], er);
                     const Limbs58 x = to_limbs58(ps[s], er);
-                    ls[s] = Limbs58{-x.h, -x.l};
+                    ls[s] = Limbs58{opaque(-x.h), opaque(-x.l)};
                     if (s < M - 1) pe[s] *= kE[s];
                 }
             }
@@ -209,10 +209,10 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
                         E[s] = pe[s] * xe;                     // (2 beta_a rho_a + rho_dot_a) e_a; not used for the last
                         const Limbs58 l = to_limbs58(xe, exc), m{__double2hiint(xs), __double2loint(xs)};
                         long long hi = 0, mid = 0;
-                        fma_limbs58(hi, mid, le[s].h, le[s].l, l);
-                        fma_limbs58(hi, mid, ls[s].h, ls[s].l, m);
+                        fma_limbs58(hi, mid, le[s], l);
+                        fma_limbs58(hi, mid, ls[s], m);
                         const long long d = hi + (mid >> 29);  // below 2^59
-                        D[s] = Limbs58{(int)(d >> 29), (int)((unsigned)d & 0x1fffffffu)};
+                        D[s] = limbs_of(d);
                     }
                     const int e = er + exc - 2044 + mc.mix_exp;
                     const bool nan = er == 0x7ff || exc == 0x7ff;      // an infinite or NaN factor
@@ -221,7 +221,7 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
                         long long hi = 0, mid = 0;
 #pragma unroll
                         for (int b = 0; b < M; ++b)
-                            if (b != s) fma_limbs58(hi, mid, mc.mixh[s][b], mc.mixl[s][b], D[b]);
+                            if (b != s) fma_limbs58(hi, mid, limbs_of(mc.mix[s][b]), D[b]);
                         F[s] = double_of_int64(hi + (mid >> 29), e);
                         if (nan) F[s] = __longlong_as_double(0x7ff8000000000000ll);
                     }

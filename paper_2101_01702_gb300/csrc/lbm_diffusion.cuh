@@ -218,14 +218,14 @@ __device__ __forceinline__ void diffusion_refined(const MechConst &mc, const dou
             const int e = (__float_as_int(x[s]) >> 23) & 0xff, f = min(max(e - e0, 0), 41);
             int xi = __float2int_rn(x[s] * pow2f(kx - f));
             const long long v = ln[s * bs];
-            long long ph = (long long)(int)(v >> 32) * xi, pl = (long long)(int)v * xi;
+            long long ph = (long long)opaque((int)(v >> 32)) * xi, pl = (long long)opaque((int)v) * xi;
             if (f > 0 && (f > 40 || ((ph < 0 ? -ph : ph) >> (58 - f)) != 0)) {
                 xi = 0;
                 ph = pl = 0;
             }
             const long long p = f == 0 ? (ph >> 1) + (pl >> 30)
                                        : (ph << (f - 1)) + (f <= 30 ? pl >> (30 - f) : pl << (f - 30));
-            w[s] = Limbs58{(int)(p >> 29), (int)((unsigned)p & 0x1fffffffu)};
+            w[s] = limbs_of(p);
             x[s] = (float)xi * pow2f(f - kx);
         }
         float r[M];
@@ -234,7 +234,7 @@ __device__ __forceinline__ void diffusion_refined(const MechConst &mc, const dou
             long long hi = 0, mid = 0;
 #pragma unroll
             for (int b = 0; b < M; ++b)
-                if (b != s) fma_limbs58(hi, mid, mc.mixh[s][b], mc.mixl[s][b], w[b]);
+                if (b != s) fma_limbs58(hi, mid, limbs_of(mc.mix[s][b]), w[b]);
             const long long G = hi + (mid >> 29);
             // G as a pair of floats, from pieces of 22, 23 and 18 bits
             const float G1 = (__int_as_float(0x4b400000 + (int)(G >> 41)) - 12582912.0f) * g1;

@@ -101,6 +101,10 @@ __host__ __device__ constexpr size_t ghost_bytes_for(int S, size_t plane, int nl
 //   g_a/(R_U T) = gco0 (1 - ln T) + gco1 T + gco2 T^2 + gco3 T^3 + gco4 T^4
 //                 + gco5 / T + gco6
 // Both the constant-cp and the 7-coefficient thermodynamics map onto these.
+struct alignas(8) MixLimbs {
+    int h, l;
+};
+
 struct MechConst {
     int M, R;
     int visc_model;
@@ -110,14 +114,14 @@ struct MechConst {
     double hco[LBMK_MAXM][6], uco[LBMK_MAXM][6], gco[LBMK_MAXM][7];
     double inv_WWD[LBMK_MAXM][LBMK_MAXM];                   // 1 / (W_a W_b D_ab), 0 on the diagonal
     float inv_WWD_f[LBMK_MAXM][LBMK_MAXM];
-    // 1/D_ab as the integer mixh 2^29 + mixl < 2^58, in units of 2^mix_exp
+    // 1/D_ab as the integer mix.h 2^29 + mix.l < 2^58, in units of 2^mix_exp
     // (mix_fixed: every entry exact, see lbm_pack_tables; at most LBMK_MIXM
     // species, so that four slots fit constant memory); 0 on the diagonal;
     // 1/W_a and 1/D_ab as pairs of floats
     int mix_fixed, mix_exp;
     float invW_h[LBMK_MAXM], invW_l[LBMK_MAXM];
     float invD_h[LBMK_MIXM][LBMK_MIXM], invD_l[LBMK_MIXM][LBMK_MIXM];
-    int mixh[LBMK_MIXM][LBMK_MIXM], mixl[LBMK_MIXM][LBMK_MIXM];
+    MixLimbs mix[LBMK_MIXM][LBMK_MIXM];
     int rtype[LBMK_MAXR], rev[LBMK_MAXR];
     int nreac[LBMK_MAXR], nprod[LBMK_MAXR];
     int reac[LBMK_MAXR][3], prod[LBMK_MAXR][3];             // species of each molecule

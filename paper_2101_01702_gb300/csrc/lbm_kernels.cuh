@@ -1095,15 +1095,17 @@ __device__ __forceinline__ double exp_table(double x)
     const u64 xm = sh >= 0 ? m << sh : m >> (sh < -63 ? 63 : -sh);
     const u64 xs = hi < 0 ? 0ull - xm : xm;
     const i64 r = (i64)(xs - (u64)(i64)n * (u64)L1 - (u64)(((i64)n * L2) >> 18));
-    const int rh = (int)(r >> 32), rl = (int)((unsigned)r >> 1);
+    const int rh = opaque((int)(r >> 32)), rl = opaque((int)((unsigned)r >> 1));
     const i64 r2 = (i64)rh * rh + (((i64)rh * rl) >> 30);                   // units of 2^-76
-    const int t = (int)(2147483648.0 / 6) + (int)(((i64)rh * (int)(2147483648.0 / 24)) >> 38) +
-                  (int)(((i64)(int)(r2 >> 32) * (int)(2147483648.0 / 120)) >> 44);
-    const int rt = (int)(((i64)rh * t) >> 27);                              // r t, units of 2^-42
-    const i64 p = r + (r2 >> 7) + (((i64)(int)(r2 >> 27) * rt) >> 21);      // e^r - 1, units of 2^-70
+    const int t = opaque((int)(2147483648.0 / 6) + (int)(((i64)rh * (int)(2147483648.0 / 24)) >> 38) +
+                         (int)(((i64)opaque((int)(r2 >> 32)) * (int)(2147483648.0 / 120)) >> 44));
+    const int rt = opaque((int)(((i64)rh * t) >> 27));                      // r t, units of 2^-42
+    // e^r - 1, units of 2^-70
+    const i64 p = r + (r2 >> 7) + (((i64)opaque((int)(r2 >> 27)) * rt) >> 21);
     const u64 tb = (u64)__double_as_longlong(__ldg(&c_exp2_256[n & 255]));
     const u64 tm = (tb & 0xfffffffffffffull) | 0x10000000000000ull;         // 2^(j/256), units of 2^-52
-    const int th = (int)(tm >> 22), tl = (int)(tm & 0x3fffffull), ph = (int)(p >> 32), pl = (int)((unsigned)p >> 1);
+    const int th = opaque((int)(tm >> 22)), tl = opaque((int)(tm & 0x3fffffull));
+    const int ph = opaque((int)(p >> 32)), pl = opaque((int)((unsigned)p >> 1));
     const i64 tp = (i64)th * ph + (((i64)th * pl) >> 31) + (((i64)tl * ph) >> 22);
     u64 y = (tm << 10) + (u64)(tp >> 6);                                    // units of 2^-62
     const int lead = (int)(y >> 62), d = (lead >= 2) - (lead == 0);         // y in [1/2, 4): one place up or down

@@ -95,8 +95,8 @@ static inline int lbm_pack_tables(const lbm_species *sp, const lbm_mechanism *me
             for (int b = 0; b < M; ++b)
                 if (a != b) {
                     const long long v = (long long)ldexp(1.0 / sp->D[M * a + b], 57 - e);
-                    mc.mixh[a][b] = (int)(v >> 29);
-                    mc.mixl[a][b] = (int)(v & 0x1fffffff);
+                    mc.mix[a][b].h = (int)(v >> 29);
+                    mc.mix[a][b].l = (int)(v & 0x1fffffff);
                     mc.invD_h[a][b] = (float)(1.0 / sp->D[M * a + b]);
                     mc.invD_l[a][b] = (float)(1.0 / sp->D[M * a + b] - (double)mc.invD_h[a][b]);
                 }

@@ -148,7 +148,7 @@ int main(int argc, char **argv)
         long long hi = 0, mid = 0;
         Q ref = 0, big = 0;
         for (int b = 1; b < M; ++b) {
-            fma_limbs58(hi, mid, mc.mixh[0][b], mc.mixl[0][b], to_limbs58(v[b], e));
+            fma_limbs58(hi, mid, limbs_of(mc.mix[0][b]), to_limbs58(v[b], e));
             const double k = 1.0 / D[b];
             ref += (Q)k * v[b];
             big = max((double)big, 0.0) > fabs((double)(k * v[b])) ? big : (Q)fabs((double)(k * v[b]));
