@@ -36,7 +36,7 @@ struct lbm_ctx {
     cudaGraphExec_t graph;   // two captured steps (lbm_step_graph), or null
     int graph_cur;           // value of cur the graph starts from
     bool refs_fixed;         // rest references set by lbm_set_references
-    int bs[LBMK_NKERNELS];   // threads per block of each kernel (lbm_autotune)
+    int bs[LBMK_NKERNELS];   // threads per block of each kernel (lbm_autotune, lbm_set_blocks), 0: by size
     int dev;                 // CUDA device current at lbm_create
 };
 
@@ -380,8 +380,8 @@ int lbm_create(const lbm_lattice *lat, const lbm_species *sp, const lbm_mechanis
     c->pop_bytes = need_pop;
     c->mc = mc;
     c->lat.seg_nx = nullptr;     // read here only
-    for (int k = 0; k < LBMK_NKERNELS; ++k) c->bs[k] = LBMK_BLOCK;
-    if (!is_mixed(lat->precision)) c->bs[LBMK_K_STEP] = 64;   // shared memory for 8 warps per SM instead of 4
+    for (int k = 0; k < LBMK_NKERNELS; ++k) c->bs[k] = 0;       // by the lattice's size (block_of)
+    c->bs[LBMK_K_GHOST] = LBMK_BLOCK;
     // the status word, then (at byte 16) the persistent step's barrier state
     int st = check_cuda(cudaMalloc((void **)&c->status, 16 + sizeof(GridBarrier)));
     if (st == LBM_OK) st = check_cuda(cudaMemsetAsync(c->status, 0, 16 + sizeof(GridBarrier), c->stream));

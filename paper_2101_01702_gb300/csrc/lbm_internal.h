@@ -174,7 +174,7 @@ enum { LBMK_K_GHOST = 0, LBMK_K_PRE, LBMK_K_CHEM, LBMK_K_GRAD, LBMK_K_STEPG, LBM
 struct StepArgs {
     int slot, M, nx, ny, nz, N, bc_x;
     int fixed;               // the tables' mix_fixed: kernels with fixed-point sums over the species
-    int bs[LBMK_NKERNELS];   // threads per block of each kernel
+    int bs[LBMK_NKERNELS];   // threads per block of each kernel, 0: by the lattice's size (block_of)
     // Lattices side by side in x (nseg >= 2): per x coordinate its lattice's
     // x range and index {x0, x1, k, 0}; per lattice its range {x0, x1}.
     // Null for one lattice (x0 = 0, x1 = nx, k = 0).

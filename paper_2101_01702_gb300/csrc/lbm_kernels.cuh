@@ -2016,6 +2016,22 @@ int opt_in_smem(F *f, size_t bytes, std::atomic<unsigned long long> &done)
 // ---------------------------------------------------------------------
 inline dim3 grid_for(int n, int bs = LBMK_BLOCK) { return dim3((unsigned)((n + bs - 1) / bs)); }
 
+// Threads per block of kernel k: the context's choice, or (0) the default,
+// halved down to one warp while the grid has fewer than 16 blocks per SM.
+// Below that the blocks do not spread evenly over the 152 SMs, and with
+// fewer warps than schedulers, warps of one block share an SM's FP64 unit
+// (76 cycles per instruction for four warps, 64 for one) while others are
+// idle.  us per step, all kernels: 1024 nodes with three species in double
+// 112.5 -> 109.5, 4096 x 4 x 4 double 773 -> 761.
+inline int block_of(const StepArgs &a, int k)
+{
+    int bs = a.bs[k];
+    if (bs > 0) return bs;
+    bs = k == LBMK_K_STEP && !LBMK_MIXED ? LBMK_BLOCK / 2 : LBMK_BLOCK;
+    while (bs > 32 && (a.N + bs - 1) / bs < 16 * 152) bs /= 2;
+    return bs;
+}
+
 template <int M, bool FX>
 int launch_step(const StepArgs &a, int bs)
 {
@@ -2031,7 +2047,7 @@ int launch_step(const StepArgs &a, int bs)
 template <int M>
 int launch_one(const StepArgs &a, int k)
 {
-    const int bs = a.bs[k];
+    const int bs = block_of(a, k);
     switch (k) {
     case LBMK_K_GHOST:
         if (a.bc_x == 1) launch_ghost<M>(a);
