@@ -65,7 +65,7 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
             Rw[s] = rho * ld(rr.y + s);
             conc[s] = Rw[s] * mc.invW[s];
         }
-        molar_production<M>(mc, T, conc, sh, sh + M * bs, sh + 2 * M * bs, t, bs);
+        production_rates<M>(mc, T, conc, sh, sh + M * bs, sh + 2 * M * bs, t, bs);
         const double kappa = ld(rr.kappa);
 #pragma unroll
         for (int s = 0; s < M; ++s) {

@@ -30,29 +30,6 @@
 
 namespace {
 
-// a + b as a rounded sum and its error (Knuth).
-__device__ __forceinline__ float two_sum(float a, float b, float &err)
-{
-    const float s = a + b, bb = s - a;
-    err = (a - (s - bb)) + (b - bb);
-    return s;
-}
-
-// The leading 24 and the next 23 bits of d as floats (0 below the float
-// range; d within it above).
-__device__ __forceinline__ void split2(double d, float &h, float &l)
-{
-    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-    const int ed = (int)((hi >> 20) & 0x7ffu) - 896;                 // float exponent field
-    const unsigned sign = hi & 0x80000000u;
-    const unsigned man = ((hi & 0xfffffu) << 3) | (lo >> 29);
-    const bool ok = ed > 24;
-    h = ok ? __uint_as_float(sign | ((unsigned)ed << 23) | man) : 0.0f;
-    // 23 of the low 29 bits as a float of exponent ed - 23, less its implicit one
-    const unsigned e2 = sign | ((unsigned)(ed - 23) << 23);
-    l = ok ? __uint_as_float(e2 | ((lo & 0x1fffffffu) >> 6)) - __uint_as_float(e2) : 0.0f;
-}
-
 // 2^k, clamped to the normal floats.
 __device__ __forceinline__ float pow2f(int k)
 {

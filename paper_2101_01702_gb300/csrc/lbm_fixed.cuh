@@ -83,4 +83,30 @@ __device__ __forceinline__ double double_of_int64(long long s, int e)
     return __longlong_as_double((long long)bits);
 }
 
+// a + b as a rounded sum and its error (Knuth).
+__device__ __forceinline__ float two_sum(float a, float b, float &err)
+{
+    const float s = a + b, bb = s - a;
+    err = (a - (s - bb)) + (b - bb);
+    return s;
+}
+
+// The leading 24 and the next 23 bits of d as floats; d rounded to float and 0
+// outside the range where both are normal (and not zero).
+__device__ __forceinline__ void split2(double d, float &h, float &l)
+{
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const int ed = (int)((hi >> 20) & 0x7ffu) - 896;                 // float exponent field
+    const unsigned sign = hi & 0x80000000u;
+    if (ed > 24 && ed < 255) {
+        h = __uint_as_float(sign | ((unsigned)ed << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+        // 23 of the low 29 bits as a float of exponent ed - 23, less its implicit one
+        const unsigned e2 = sign | ((unsigned)(ed - 23) << 23);
+        l = __uint_as_float(e2 | ((lo & 0x1fffffffu) >> 6)) - __uint_as_float(e2);
+    } else {
+        h = (hi << 1 | lo) == 0u ? 0.0f : __double2float_rn(d);
+        l = 0.0f;
+    }
+}
+
 }  // namespace

@@ -105,6 +105,15 @@ struct alignas(8) MixLimbs {
     int h, l;
 };
 
+// The exponent of a reaction's rate coefficient in fixed point: ln A in units
+// of 2^-53, b and theta as limbs in units of 2^bx_exp and 2^tx_exp, and all as
+// floats.
+struct RateLimbs {
+    long long log_A;
+    MixLimbs b, theta;
+    float log_Af, bf, thetaf;
+};
+
 struct MechConst {
     int M, R;
     int visc_model;
@@ -128,14 +137,23 @@ struct MechConst {
     int dn[LBMK_MAXR];                                      // sum of product minus reactant coefficients
     double log_A[LBMK_MAXR], b[LBMK_MAXR], theta[LBMK_MAXR];
     double dlow[LBMK_MAXR][3];                              // falloff: ln(A0/A), b0 - b, theta0 - theta
-    double eff[LBMK_MAXR][LBMK_MAXM];
+    double eff[LBMK_MAXR][LBMK_MIXM];
+    // Fixed-point exponents (molar_production_fixed; chem_fixed: the tables
+    // are in range): gco in limbs, units of 2^gx_exp[j] (j < 6; gx_mask: which
+    // j any species has), gx0 = gco6 in units of 2^-53, all as floats
+    int chem_fixed, gx_mask, gx_exp[6], bx_exp, tx_exp;
+    double r_over_P0;
+    long long gx0[LBMK_MIXM];
+    MixLimbs gx[LBMK_MIXM][6];
+    float gxf[LBMK_MIXM][7];
+    RateLimbs rx[LBMK_MAXR];
     // Mixture-averaged transport (transport = 1): species viscosity law,
     // Wilke's mass factors wq[a][b] = (W_b/W_a)^(1/4) and
     // wd[a][b] = (8 (1 + W_a/W_b))^(-1/2), 5/4 R_a for Eucken's relation, and
     // the diffusivity law (T/T_tr)^D_exp (P_tr/P).
     int transport;
     double mu0[LBMK_MAXM], mu_exp[LBMK_MAXM], eucken[LBMK_MAXM];
-    double wq[LBMK_MAXM][LBMK_MAXM], wd[LBMK_MAXM][LBMK_MAXM];
+    double wq[LBMK_MIXM][LBMK_MIXM], wd[LBMK_MIXM][LBMK_MIXM];
     double log_T_tr, D_exp, P_tr;
     // Mixed precision: stored float value = population - ref[s][i] for the
     // moving directions of the species and mixture sets (s < M); ref is a
@@ -165,6 +183,8 @@ inline void lbmk_reference_moments(MechConst &mc, int M)
 }
 
 #define LBMK_BLOCK 128      // default block; the block of k_pre and k_step is at most this
+static_assert(LBMK_SLOTS * sizeof(MechConst) <= 65536, "four slots have to fit constant memory");
+
 #define LBMK_MAXBLOCK 256   // largest block of the kernels tuned up to it (k_grad, k_step_g; k_chem)
 
 // The kernels of one step, in launch order (timing phases and autotuned

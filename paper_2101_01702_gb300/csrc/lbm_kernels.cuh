@@ -1056,6 +1056,31 @@ __device__ const double c_exp2_256[256] = {
     0x1.fa7c1819e90d8p+0, 0x1.fbdba3692d514p+0, 0x1.fd3c22b8f71f1p+0, 0x1.fe9d96b2a23d9p+0,
 };
 
+// e^(x - N ln2/256) 2^(N/256) for x in units of 2^-70, modulo 2^64, and N = n
+// (see exp_table; ln2/256 as L1 2^-70 + L2 2^-88).
+__device__ __forceinline__ double exp_reduced(unsigned long long xs, int n, long long L1, long long L2)
+{
+    typedef long long i64;
+    typedef unsigned long long u64;
+    const i64 r = (i64)(xs - (u64)(i64)n * (u64)L1 - (u64)(((i64)n * L2) >> 18));
+    const int rh = opaque((int)(r >> 32)), rl = opaque((int)((unsigned)r >> 1));
+    const i64 r2 = (i64)rh * rh + (((i64)rh * rl) >> 30);                   // units of 2^-76
+    const int t = opaque((int)(2147483648.0 / 6) + (int)(((i64)rh * (int)(2147483648.0 / 24)) >> 38) +
+                         (int)(((i64)opaque((int)(r2 >> 32)) * (int)(2147483648.0 / 120)) >> 44));
+    const int rt = opaque((int)(((i64)rh * t) >> 27));                      // r t, units of 2^-42
+    // e^r - 1, units of 2^-70
+    const i64 p = r + (r2 >> 7) + (((i64)opaque((int)(r2 >> 27)) * rt) >> 21);
+    const u64 tb = (u64)__double_as_longlong(__ldg(&c_exp2_256[n & 255]));
+    const u64 tm = (tb & 0xfffffffffffffull) | 0x10000000000000ull;         // 2^(j/256), units of 2^-52
+    const int th = opaque((int)(tm >> 22)), tl = opaque((int)(tm & 0x3fffffull));
+    const int ph = opaque((int)(p >> 32)), pl = opaque((int)((unsigned)p >> 1));
+    const i64 tp = (i64)th * ph + (((i64)th * pl) >> 31) + (((i64)tl * ph) >> 22);
+    u64 y = (tm << 10) + (u64)(tp >> 6);                                    // units of 2^-62
+    const int lead = (int)(y >> 62), d = (lead >= 2) - (lead == 0);         // y in [1/2, 4): one place up or down
+    y >>= 9 + d;
+    return __longlong_as_double((i64)(((u64)(unsigned)(1022 + (n >> 8) + d) << 52) + (y >> 1) + (y & 1)));
+}
+
 // exp(x) by the table-driven method of P. T. P. Tang (ACM Trans. Math.
 // Softw. 15(2), 1989): x = (256 m + j) ln2/256 + r with |r| <= 1.04 ln2/512,
 // so exp(x) = 2^m 2^(j/256) e^r, and e^r - 1 is its degree-5 Taylor
@@ -1079,7 +1104,6 @@ __device__ __forceinline__ double exp_table(double x)
 {
     constexpr double kInv = 0x1.71547652b82fep+8, kL1 = 0x1.62e42fefc0000p-9, kL2 = -0x1.c610ca86c3899p-45;
     constexpr long long L1 = (long long)(kL1 * 0x1p+70), L2 = (long long)(kL2 * 0x1p+88);
-    typedef long long i64;
     typedef unsigned long long u64;
     const int hi = __double2hiint(x);
     const unsigned lo = (unsigned)__double2loint(x), mag = (unsigned)hi & 0x7fffffffu;
@@ -1093,24 +1117,7 @@ __device__ __forceinline__ double exp_table(double x)
     const u64 m = ((u64)((mag & 0xfffffu) | 0x100000u) << 32) | lo;
     const int sh = ed - 1005;
     const u64 xm = sh >= 0 ? m << sh : m >> (sh < -63 ? 63 : -sh);
-    const u64 xs = hi < 0 ? 0ull - xm : xm;
-    const i64 r = (i64)(xs - (u64)(i64)n * (u64)L1 - (u64)(((i64)n * L2) >> 18));
-    const int rh = opaque((int)(r >> 32)), rl = opaque((int)((unsigned)r >> 1));
-    const i64 r2 = (i64)rh * rh + (((i64)rh * rl) >> 30);                   // units of 2^-76
-    const int t = opaque((int)(2147483648.0 / 6) + (int)(((i64)rh * (int)(2147483648.0 / 24)) >> 38) +
-                         (int)(((i64)opaque((int)(r2 >> 32)) * (int)(2147483648.0 / 120)) >> 44));
-    const int rt = opaque((int)(((i64)rh * t) >> 27));                      // r t, units of 2^-42
-    // e^r - 1, units of 2^-70
-    const i64 p = r + (r2 >> 7) + (((i64)opaque((int)(r2 >> 27)) * rt) >> 21);
-    const u64 tb = (u64)__double_as_longlong(__ldg(&c_exp2_256[n & 255]));
-    const u64 tm = (tb & 0xfffffffffffffull) | 0x10000000000000ull;         // 2^(j/256), units of 2^-52
-    const int th = opaque((int)(tm >> 22)), tl = opaque((int)(tm & 0x3fffffull));
-    const int ph = opaque((int)(p >> 32)), pl = opaque((int)((unsigned)p >> 1));
-    const i64 tp = (i64)th * ph + (((i64)th * pl) >> 31) + (((i64)tl * ph) >> 22);
-    u64 y = (tm << 10) + (u64)(tp >> 6);                                    // units of 2^-62
-    const int lead = (int)(y >> 62), d = (lead >= 2) - (lead == 0);         // y in [1/2, 4): one place up or down
-    y >>= 9 + d;
-    return __longlong_as_double((i64)(((u64)(unsigned)(1022 + (n >> 8) + d) << 52) + (y >> 1) + (y & 1)));
+    return exp_reduced(hi < 0 ? 0ull - xm : xm, n, L1, L2);
 }
 
 // Exponential of the rate expressions: exp_table(), except in the fast mixed
@@ -1133,6 +1140,172 @@ __device__ __forceinline__ double exp_rate(double x)
     return exp_table(x);
 #endif
 }
+
+#if !LBMK_FAST
+// exp(x) for x in units of 2^-53 (modulo 2^64) and a float within 1e-4 of it;
+// beyond +-707 from the float alone.
+__device__ __forceinline__ double exp_fixed(long long x, float xf)
+{
+    constexpr double kInv = 0x1.71547652b82fep+8, kL1 = 0x1.62e42fefc0000p-9, kL2 = -0x1.c610ca86c3899p-45;
+    constexpr long long L1 = (long long)(kL1 * 0x1p+70), L2 = (long long)(kL2 * 0x1p+88);
+    if (!(fabsf(xf) < 707.0f)) return exp((double)xf);
+    const int n = __float_as_int(fmaf(xf, (float)kInv, 12582912.0f)) - 0x4b400000;
+    return exp_reduced((unsigned long long)x << 17, n, L1, L2);
+}
+
+// v 2^sh modulo 2^64 (sh within +-63; smaller gives the sign).
+__device__ __forceinline__ long long shift_by(long long v, int sh)
+{
+    return sh >= 0 ? (long long)((unsigned long long)v << (sh & 63)) : v >> (sh < -63 ? 63 : -sh);
+}
+
+// Sums of the molar production rates, one 8-byte column per species: in
+// double, or (PAIR) in pairs of floats, for callers that store the rates as
+// floats: a sum and the sum of its rounding errors (two_sum), 48 bits.
+template <bool PAIR>
+struct RateSums {
+    double *col;
+    int stride;
+    __device__ __forceinline__ void clear(int s) { col[s * stride] = 0.0; }
+    struct Term {
+        double q;
+        float h, l;
+    };
+    __device__ __forceinline__ Term term(double q) const
+    {
+        Term t{q, 0.0f, 0.0f};
+        if (PAIR) split2(q, t.h, t.l);
+        return t;
+    }
+    template <int SIGN>
+    __device__ __forceinline__ void add(int s, const Term &t)
+    {
+        if (PAIR) {
+            float2 *p = reinterpret_cast<float2 *>(col + s * stride);
+            float2 v = *p;
+            float e;
+            v.x = two_sum(v.x, SIGN * t.h, e);
+            v.y += e + SIGN * t.l;
+            *p = v;
+        } else {
+            col[s * stride] += SIGN * t.q;
+        }
+    }
+    // w_s times the molar mass
+    __device__ __forceinline__ double mass(int s, double W) const { return W * col[s * stride]; }
+    __device__ __forceinline__ float mass_float(int s, double W) const
+    {
+        const float2 v = *reinterpret_cast<const float2 *>(col + s * stride);
+        float wh, wl;
+        split2(W, wh, wl);
+        const float p = wh * v.x;
+        return p + (fma(wh, v.x, -p) + fma(wh, v.y, wl * v.x));
+    }
+};
+
+// Molar production rates as molar_production below forms them, with every
+// exponent an integer sum in units of 2^-53: the Gibbs functions
+//   g_a/(R_U T) = sum_j gco_aj phi_j,  phi = 1 - ln T, T .. T^4, 1/T, 1,
+// and ln k_f - sum_reac g, from products of 58-bit limbs (each phi_j with
+// its leading bit at 2^57, the coefficients of a j relative to the largest)
+// brought to that unit, and a float beside each exponent for exp_fixed's
+// range reduction.  A sum of these is good to a few units of 2^-52; in
+// double it carried half a unit of the largest partial sum, 2^-47 at the
+// exponents of 300 K.  146 FP64 operations per node of nine species and 21
+// reactions leave the FP64 pipe, and 80 more where the rates are summed in
+// pairs of floats (RateSums).  For tables in range (MechConst::chem_fixed).
+template <int M, bool PAIR>
+__device__ __forceinline__ void molar_production_fixed(const MechConst &mc, double T, const double *conc,
+                                                       double *sh_act, double *sh_g, RateSums<PAIR> w, int t,
+                                                       int stride)
+{
+    typedef long long i64;
+    const double invT = 1.0 / T, lnT = log(T), lnTr = lnT - mc.log_T_ref;
+    Limbs58 P[6], Ll, Il;
+    int sp[6], sb, st;
+    float pf[6];
+    {
+        const double T2 = T * T;
+        const double phi[6] = {1.0 - lnT, T, T2, T2 * T, T2 * T2, invT};
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            const int e = biased_exponent(phi[j]);
+            P[j] = to_limbs58(phi[j], e);
+            sp[j] = mc.gx_exp[j] + e - 969;
+            pf[j] = d2f(phi[j]);
+        }
+        const int eL = biased_exponent(lnTr), eI = biased_exponent(invT);
+        Ll = to_limbs58(lnTr, eL);
+        Il = P[5];
+        sb = mc.bx_exp + eL - 969;
+        st = mc.tx_exp + eI - 969;
+    }
+    const float lf = d2f(lnTr);
+    i64 *gx = reinterpret_cast<i64 *>(sh_g);
+#pragma unroll 1
+    for (int s = 0; s < M; ++s) {
+        i64 g = mc.gx0[s];
+        float gf = mc.gxf[s][6];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            if (!(mc.gx_mask >> j & 1)) continue;          // no species has the term
+            i64 hi = 0, mid = 0;
+            fma_limbs58(hi, mid, limbs_of(mc.gx[s][j]), P[j]);
+            g += shift_by(hi + (mid >> 29), sp[j]);
+            gf = fmaf(mc.gxf[s][j], pf[j], gf);
+        }
+        // beyond the range of the unit: e^g is 0 or infinite either way
+        if (!(fabsf(gf) < 1000.0f)) g = gf < 0.0f ? -(1000ll << 53) : 1000ll << 53;
+        gx[s * stride + t] = g;
+        sh_act[s * stride + t] = conc[s] * exp_fixed(g, gf);
+        w.clear(s);
+    }
+    const double c0 = mc.P0_over_r * invT, ic0 = T * mc.r_over_P0;   // P0/(r T) and its inverse
+#pragma unroll 1
+    for (int k = 0; k < mc.R; ++k) {
+        const int nr = mc.nreac[k], np = mc.nprod[k];     // nr >= 1 (checked at packing)
+        // exponent ln k_f - sum_reac g
+        const RateLimbs &rx = mc.rx[k];
+        i64 bh = 0, bm = 0, th = 0, tm = 0;
+        fma_limbs58(bh, bm, limbs_of(rx.b), Ll);
+        fma_limbs58(th, tm, limbs_of(rx.theta), Il);
+        i64 arg = rx.log_A + shift_by(bh + (bm >> 29), sb) - shift_by(th + (tm >> 29), st);
+        float af = fmaf(rx.bf, lf, fmaf(-rx.thetaf, pf[5], rx.log_Af));
+        double p = 1.0;
+        for (int j = 0; j < nr; ++j) {
+            const int sidx = mc.reac[k][j] * stride + t;
+            const i64 g = gx[sidx];
+            arg -= g;
+            af -= (float)(int)(g >> 32) * 0x1p-21f;
+            p = j == 0 ? sh_act[sidx] : p * sh_act[sidx];
+        }
+        if (mc.rev[k]) {
+            double pr = np > 0 ? sh_act[mc.prod[k][0] * stride + t] : 1.0;
+            for (int j = 1; j < np; ++j) pr *= sh_act[mc.prod[k][j] * stride + t];
+            const int dn = mc.dn[k];
+            for (int j = 0; j < dn; ++j) pr *= ic0;
+            for (int j = 0; j < -dn; ++j) pr *= c0;
+            p -= pr;
+        }
+        double q = p * exp_fixed(arg, af);
+        const int type = mc.rtype[k];
+        if (type != 0) {
+            double cM = 0.0;
+#pragma unroll
+            for (int s = 0; s < M; ++s) cM = fma(mc.eff[k][s], conc[s], cM);
+            if (type == 1) {
+                q *= cM;
+            } else {
+                const double Pr = exp_table(fma(mc.dlow[k][1], lnTr, fma(-mc.dlow[k][2], invT, mc.dlow[k][0]))) * cM;
+                q *= Pr / (1.0 + Pr);
+            }
+        }
+        const typename RateSums<PAIR>::Term qt = w.term(q);
+        for (int j = 0; j < nr; ++j) w.template add<-1>(mc.reac[k][j], qt);
+        for (int j = 0; j < np; ++j) w.template add<1>(mc.prod[k][j], qt);
+    }
+}
+#endif  // !LBMK_FAST
 
 // Molar production rates sum_k (nu''_ak - nu'_ak) q_k at temperature T and
 // concentrations conc, left in sh_w[a * stride + t]; sh_act and sh_g are
@@ -1190,6 +1363,20 @@ __device__ __forceinline__ void molar_production(const MechConst &mc, double T, 
         for (int j = 0; j < nr; ++j) sh_w[mc.reac[k][j] * stride + t] -= qr;
         for (int j = 0; j < np; ++j) sh_w[mc.prod[k][j] * stride + t] += qr;
     }
+}
+
+// The rates in sh_w by either form.
+template <int M>
+__device__ __forceinline__ void production_rates(const MechConst &mc, double T, const double *conc, double *sh_act,
+                                                 double *sh_g, WReal *sh_w, int t, int stride)
+{
+#if !LBMK_FAST
+    if (mc.chem_fixed) {
+        molar_production_fixed<M, false>(mc, T, conc, sh_act, sh_g, RateSums<false>{sh_w + t, stride}, t, stride);
+        return;
+    }
+#endif
+    molar_production<M>(mc, T, conc, sh_act, sh_g, sh_w, t, stride);
 }
 
 // The temperature of a node from its pulled populations, with the moments in
@@ -1282,7 +1469,7 @@ __global__ void __launch_bounds__(LBMK_BLOCK, LBMK_MOM_MINB) k_moments(StepArgs 
         double conc[M];
 #pragma unroll
         for (int s = 0; s < M; ++s) conc[s] = sh_act[s * LBMK_BLOCK + threadIdx.x] * mc.invW[s];
-        molar_production<M>(mc, T, conc, sh_act, sh_g, sh_w, threadIdx.x, LBMK_BLOCK);
+        production_rates<M>(mc, T, conc, sh_act, sh_g, sh_w, threadIdx.x, LBMK_BLOCK);
         if (mask & 128u) {
             for (int s = 0; s < M; ++s) out[(row + s) * N + n] = mc.W[s] * (double)sh_w[s * LBMK_BLOCK + threadIdx.x];
             row += M;
@@ -1838,9 +2025,19 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
         double conc[M];
 #pragma unroll
         for (int s = 0; s < M; ++s) conc[s] = cvt<double>(rho) * cvt<double>(Yl[s]) * mc.invW[s];
-        molar_production<M>(mc, ldd(DR_T), conc, sh_act, sh_g, sh_w, threadIdx.x, bs);
+#if !LBMK_FAST
+        if (mc.chem_fixed) {
+            const RateSums<true> w{sh_w + threadIdx.x, bs};
+            molar_production_fixed<M, true>(mc, ldd(DR_T), conc, sh_act, sh_g, w, threadIdx.x, bs);
 #pragma unroll
-        for (int s = 0; s < M; ++s) wd[s] = cvt<Real>(mc.W[s] * sh_w[s * bs + threadIdx.x]);
+            for (int s = 0; s < M; ++s) wd[s] = w.mass_float(s, mc.W[s]);
+        } else
+#endif
+        {
+            molar_production<M>(mc, ldd(DR_T), conc, sh_act, sh_g, sh_w, threadIdx.x, bs);
+#pragma unroll
+            for (int s = 0; s < M; ++s) wd[s] = cvt<Real>(mc.W[s] * sh_w[s * bs + threadIdx.x]);
+        }
     }
     const Real u2[3] = {u[0] * u[0], u[1] * u[1], u[2] * u[2]};
 
@@ -2545,7 +2742,7 @@ __global__ void __launch_bounds__(LBMK_BLOCK) k_chem_at(StepArgs a, int n, const
     }
     const double T = T_in[i];
     if (rho_dot) {
-        molar_production<M>(mc, T, conc, sh_act, sh_g, sh_w, t, LBMK_BLOCK);
+        production_rates<M>(mc, T, conc, sh_act, sh_g, sh_w, t, LBMK_BLOCK);
 #pragma unroll
         for (int s = 0; s < M; ++s) rho_dot[(size_t)s * n + i] = mc.W[s] * (double)sh_w[s * LBMK_BLOCK + t];
     }

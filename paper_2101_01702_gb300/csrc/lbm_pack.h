@@ -8,6 +8,57 @@
 #include "../../include/lbm.h"
 #include "lbm_internal.h"
 
+// v[0..n) (elements `step` doubles apart) as integers below 2^58 in units of
+// 2^*e, the largest with its leading bit at 2^57.
+static inline bool lbm_pack_limbs(const double *v, int step, int n, MixLimbs *out, int out_step, size_t out_bytes,
+                                  int *e)
+{
+    double top = 0.0;
+    for (int i = 0; i < n; ++i) {
+        if (!isfinite(v[(size_t)i * step])) return false;
+        top = fmax(top, fabs(v[(size_t)i * step]));
+    }
+    *e = (top > 0.0 ? ilogb(top) : 0) - 57;
+    for (int i = 0; i < n; ++i) {
+        const long long x = (long long)ldexp(v[(size_t)i * step], -*e);
+        MixLimbs *o = (MixLimbs *)((char *)out + (size_t)i * out_step * out_bytes);
+        o->h = (int)(x >> 29);
+        o->l = (int)(x & 0x1fffffff);
+    }
+    return *e > -900 && *e < 900;
+}
+
+// The fixed-point exponents of the rates (MechConst::chem_fixed says whether
+// the tables are in range: constants below 2^9, so that sums of a few terms
+// stay within the 2^10 that the unit 2^-53 leaves).
+static inline void lbm_pack_exponents(MechConst &mc)
+{
+    bool ok = true;
+    mc.gx_mask = 0;
+    for (int j = 0; j < 6; ++j) {
+        ok &= lbm_pack_limbs(&mc.gco[0][j], 7, mc.M, &mc.gx[0][j], 6, sizeof(MixLimbs), &mc.gx_exp[j]);
+        for (int s = 0; s < mc.M; ++s)
+            if (mc.gco[s][j] != 0.0) mc.gx_mask |= 1 << j;
+    }
+    for (int s = 0; s < mc.M; ++s) {
+        ok &= fabs(mc.gco[s][6]) < 512.0;
+        mc.gx0[s] = ok ? (long long)ldexp(mc.gco[s][6], 53) : 0;
+        for (int j = 0; j < 7; ++j) mc.gxf[s][j] = (float)mc.gco[s][j];
+    }
+    if (mc.R > 0) {
+        ok &= lbm_pack_limbs(mc.b, 1, mc.R, &mc.rx[0].b, 1, sizeof(RateLimbs), &mc.bx_exp);
+        ok &= lbm_pack_limbs(mc.theta, 1, mc.R, &mc.rx[0].theta, 1, sizeof(RateLimbs), &mc.tx_exp);
+    }
+    for (int k = 0; k < mc.R; ++k) {
+        ok &= fabs(mc.log_A[k]) < 512.0;
+        mc.rx[k].log_A = ok ? (long long)ldexp(mc.log_A[k], 53) : 0;
+        mc.rx[k].log_Af = (float)mc.log_A[k];
+        mc.rx[k].bf = (float)mc.b[k];
+        mc.rx[k].thetaf = (float)mc.theta[k];
+    }
+    mc.chem_fixed = ok;
+}
+
 // Returns LBM_OK or LBM_ERR_ARG; fills mc (refs are left zero).
 static inline int lbm_pack_tables(const lbm_species *sp, const lbm_mechanism *mech, MechConst &mc)
 {
@@ -15,6 +66,7 @@ static inline int lbm_pack_tables(const lbm_species *sp, const lbm_mechanism *me
     if (!sp || !mech) return LBM_ERR_ARG;
     const int M = sp->M;
     if (M < 2 || M > LBMK_MAXM || !sp->W || !sp->D) return LBM_ERR_ARG;
+    if (M > LBMK_MIXM) return LBM_ERR_UNSUPPORTED;      // the tables below; no kernel takes more
     if (sp->thermo == LBM_THERMO_CONST_CP && (!sp->cp_R || !sp->h_form)) return LBM_ERR_ARG;
     if (sp->thermo == LBM_THERMO_POLY7 && !sp->poly7) return LBM_ERR_ARG;
     if (sp->thermo != LBM_THERMO_CONST_CP && sp->thermo != LBM_THERMO_POLY7) return LBM_ERR_ARG;
@@ -149,6 +201,8 @@ static inline int lbm_pack_tables(const lbm_species *sp, const lbm_mechanism *me
     }
     if (need_P0 && !(mech->P0 > 0)) return LBM_ERR_ARG;
     mc.P0_over_r = need_P0 ? mech->P0 / sp->r_lat : 1.0;
+    mc.r_over_P0 = 1.0 / mc.P0_over_r;
+    lbm_pack_exponents(mc);
     return LBM_OK;
 }
 

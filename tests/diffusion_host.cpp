@@ -27,6 +27,7 @@ static inline double __longlong_as_double(long long v) { return bits<double>(v);
 static inline float __uint_as_float(unsigned v) { return bits<float>(v); }
 static inline float __int_as_float(int v) { return bits<float>(v); }
 static inline int __float_as_int(float v) { return bits<int>(v); }
+static inline float __double2float_rn(double v) { return (float)v; }
 static inline int __float2int_rn(float v) { return (int)nearbyintf(v); }
 static inline bool finite_bits(float x) { return (bits<int>(x) & 0x7f800000) != 0x7f800000; }
 
