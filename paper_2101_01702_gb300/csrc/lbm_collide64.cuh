@@ -27,8 +27,7 @@ namespace {
 
 // Columns of shared memory per thread: the y factors of e and s and the x
 // factors of e as doubles, the x factors of s as limbs (FX) or doubles, for
-// c = -1, 0, 1 (12 per species); before the collision the same columns are
-// the scratch of the production rates.
+// c = -1, 0, 1 (12 per species).
 template <int M>
 constexpr int step_cols() { return 12 * M; }
 
@@ -38,8 +37,7 @@ struct PsiCoef {
 };
 __device__ __forceinline__ PsiCoef psi_coef(int c, double v)
 {
-    const double vsq = v * v;
-    return PsiCoef{c == 0 ? 1.0 - vsq : 0.5 * (c > 0 ? vsq + v : vsq - v), c == 0 ? -1.0 : 0.5};
+    return PsiCoef{c == 0 ? fma(-v, v, 1.0) : 0.5 * fma(v, v, c > 0 ? v : -v), c == 0 ? -1.0 : 0.5};
 }
 
 // FX: the tables are in the range of the fixed-point sums (MechConst::
@@ -59,28 +57,21 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
     // per species: R_b, and the factors of f_a, R_a e_a and the cross term
     double Rw[M], kf[M - 1], kE[M - 1], kF[M - 1];
     {
-        double conc[M];
-#pragma unroll
-        for (int s = 0; s < M; ++s) {
-            Rw[s] = rho * ld(rr.y + s);
-            conc[s] = Rw[s] * mc.invW[s];
-        }
-        production_rates<M>(mc, T, conc, sh, sh + M * bs, sh + 2 * M * bs, t, bs);
         const double kappa = ld(rr.kappa);
+        const double *wd = rate_rows(a, M, rec(a)) + n;
 #pragma unroll
         for (int s = 0; s < M; ++s) {
-            const double wscale = FX ? mc.invW[s] : 1.0;
-            const double ra = Rw[s];
+            const double Y = ld(rr.y + s), ra = rho * Y, wscale = FX ? mc.invW[s] : 1.0;
             // e is scaled by R_b; a species that is absent keeps a scale far
             // below every population, so that its source term survives
-            double r = FX ? conc[s] : ra;
+            double r = FX ? ra * mc.invW[s] : ra;
             r = fabs(r) < 1e-150 ? (r < 0.0 ? -1e-150 : 1e-150) : r;
             Rw[s] = r;
             if (s < M - 1) {
                 const double be = ld(rr.beta + s);
                 kf[s] = fma(-2.0, be, 1.0);
-                kE[s] = fma(2.0 * be, ra, mc.W[s] * sh[(2 * M + s) * bs + t]) / r;
-                kF[s] = (be - 1.0) * kappa * ld(rr.y + s) * wscale;
+                kE[s] = fma(2.0 * be, ra, wd[(size_t)s * N]) / r;
+                kF[s] = (be - 1.0) * kappa * Y * wscale;
             }
         }
     }

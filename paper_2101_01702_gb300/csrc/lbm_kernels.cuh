@@ -11,22 +11,24 @@
 //                  exponentials in float (see SReal, WReal, exp_rate).
 // Otherwise the moments, the temperature iteration (Eq. (temperature)),
 // the Stefan-Maxwell system (Eq. (transform1)) and the reaction rates with
-// their equilibrium constants are double precision in every unit.
+// their equilibrium constants have double precision in every unit.  The FP64
+// pipe is the scarce resource of this GPU (two multiply-adds per SM and
+// cycle): what does not need its range runs in fixed point on the integer pipe
+// or in pairs of floats (lbm_fixed.cuh), to the same accuracy.
 //
-// One time step is four launches on one stream (five with x ghosts):
+// One time step is six launches on one stream (seven with x ghosts):
 //   k_ghost  x-face ghost nodes (Sec. 5a; only for non-periodic x)
-//   k_pre    pull, all moments, Newton temperature, relaxation rates,
-//            Stefan-Maxwell diffusion velocities, the local part of the
-//            energy-flux correction and the energy equilibrium moments;
-//            writes the per-node record.
+//   k_pre    pull, all moments, Newton temperature, relaxation rates, the
+//            local part of the energy-flux correction and the energy
+//            equilibrium moments; writes the per-node record
+//   k_diff   Stefan-Maxwell diffusion velocities, beta_a
+//   k_chem   production rates of the reaction mechanism
 //   k_grad   G_alpha = (1/omega - 1/2) d_alpha Phi_alpha (Eq. (Xalpha))
 //   k_step_g pull of the energy set, sum_a H_a grad Y_a from the neighbours'
 //            records, and the collision of Eq. (g) (double)
-//   k_step   production rates of the reaction mechanism at the node
-//            (double), pull of the species and mixture sets,
-//            X = -d_alpha G_alpha from the neighbours' records, and the
-//            collisions of Eqs. (finalNumericalEquations), (f), direction
-//            by direction
+//   k_step   pull of the species and mixture sets, X = -d_alpha G_alpha from
+//            the neighbours' records, and the collisions of Eqs.
+//            (finalNumericalEquations), (f), direction by direction
 // One thread owns one lattice node; populations are structure-of-arrays
 // [set][direction][node] so that a warp's pulls are coalesced rows.
 #pragma once
@@ -80,10 +82,13 @@ typedef double WReal;
 // 128^3 double 6.71 ms at 5 + 2, 6.75 at 4 + 4, 7.21 at 2 + 3.  The species and mixture
 // collision runs fastest at 3 blocks in the mixed units (168 registers); the
 // double one (lbm_collide64.cuh) takes the registers it can get, its shared
-// memory holds it to 8 warps per SM; with the production rates inside it,
-// 256^3 mixed: 33.4 ms at 2 blocks, 27.6 ms at 3, 33.1 ms at 4.
+// memory holds it to 8 warps per SM;
+// 256^3 mixed: 15.3 ms at 2 blocks, 12.1 ms at 3, 13.6 ms at 4.
 #ifndef LBMK_PRE_MINB
 #define LBMK_PRE_MINB 5
+#endif
+#ifndef LBMK_CHEM_MINB
+#define LBMK_CHEM_MINB 4
 #endif
 #ifndef LBMK_DIFF_MINB
 #define LBMK_DIFF_MINB (LBMK_FAST ? 5 : 2)
@@ -106,12 +111,8 @@ typedef double WReal;
 // Initialisation (equilibria of every set, outside the step; FP64-bound and
 // insensitive to occupancy: 43.1-43.5 ms at 4 or 6 blocks per SM): 6 blocks
 // (80 registers, ~30 B spilled).
-// The production rates are formed inside the species collision (k_step), not
-// in a kernel of their own: they are FP64 work of the same node and overlap
-// the collision's memory traffic (256^3 mixed: k_chem 24.6 ms + k_step
-// 11.9 ms -> 29.5 ms).  The energy collision stays a kernel of its own
-// (k_step_g): inside k_step it was slower (29.5 + 4.0 ms -> 47.0 ms, more
-// spills at k_step's 168 registers).
+// The energy collision is a kernel of its own (k_step_g): inside k_step it was
+// slower (29.5 + 4.0 ms -> 47.0 ms, more spills at k_step's 168 registers).
 #ifndef LBMK_INIT_MINB
 #define LBMK_INIT_MINB 6
 #endif
@@ -562,16 +563,24 @@ __device__ __forceinline__ V psi_c(int c, V xi, V s)
 __device__ __forceinline__ void energy_moments(double rho, const double *u, double P, double hk, double rhoE,
                                                double qeq[3], double Rt[6], double &tr3)
 {
-    const double hP = hk * rho + P;
+    const double hP = fma(hk, rho, P), third = rhoE / 3.0;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         qeq[d] = hk * rho * u[d];
-        Rt[d] = hk * P + hP * u[d] * u[d] - rhoE / 3.0;
+        Rt[d] = fma(hk, P, fma(hP * u[d], u[d], -third));
     }
     Rt[3] = hP * u[0] * u[1];
     Rt[4] = hP * u[0] * u[2];
     Rt[5] = hP * u[1] * u[2];
     tr3 = (Rt[0] + Rt[1] + Rt[2]) * (1.0 / 3.0);
+}
+
+// Sums of products in the double passes are written with fma throughout: left
+// to the compiler, which products it fuses differs between builds (the
+// bounds-checked one, the persistent kernel), and so do the last bits.
+__device__ __forceinline__ double dot3(const double *a, const double *b)
+{
+    return fma(a[2], b[2], fma(a[1], b[1], a[0] * b[0]));
 }
 
 // Grad population of direction i (Eqs. (gieq), (giqeq)) for given moments.
@@ -585,7 +594,7 @@ __device__ __forceinline__ double grad_dir(int i, double rhoE, const double q[3]
     if (cx && cy) rcc += 2.0 * (cx * cy) * Rt[3];
     if (cx && cz) rcc += 2.0 * (cx * cz) * Rt[4];
     if (cy && cz) rcc += 2.0 * (cy * cz) * Rt[5];
-    return WI(i) * (rhoE + 3.0 * qc + 4.5 * (rcc - tr3));
+    return WI(i) * fma(4.5, rcc - tr3, fma(3.0, qc, rhoE));
 }
 
 // Equilibrium of every set at (rho_a, u, T), in double, handed to put(s, i, v).
@@ -599,7 +608,7 @@ __device__ void equilibria(const MechConst &mc, const double *rho_a, const doubl
 #pragma unroll
     for (int a = 0; a < M; ++a) { Y[a] = rho_a[a] / rho; inv_m += Y[a] * mc.invW[a]; }
     const double Rm = mc.r_lat * inv_m;
-    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    const double usq = dot3(u, u);
 #pragma unroll
     for (int s = 0; s < M; ++s) {
         const double zeta = (s < M - 1 ? mc.Ra[s] : Rm) * T;
@@ -934,19 +943,19 @@ __device__ __forceinline__ void ghost_warp(const StepArgs &a, int w)
 #pragma unroll
         for (int q = 0; q < 6; ++q) eu[q] = from(part[q / S], q % S);
     }
-    const double e = rhoE * ir - 0.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    const double e = fma(rhoE, ir, -0.5 * dot3(u, u));
     const double T = solve_T(eu, e, a.macro[(size_t)DR_T * a.N + n], a.status);
     if (side == 0) u[0] = u[1] = u[2] = 0.0;
     const double Rm = mc.r_lat * inv_m;
     double *gh = static_cast<double *>(a.ghost) + (size_t)gp * S * LBMK_Q * plane + yz;
     if (s < M) {
-        const double zeta = (s < M - 1 ? mc.Ra[s] : Rm) * T;
+        const double zeta = __dmul_rn(s < M - 1 ? mc.Ra[s] : Rm, T);
         const double r = s < M - 1 ? m0 : rho;
         double P3[3][3];
 #pragma unroll
         for (int d = 0; d < 3; ++d)
 #pragma unroll
-            for (int c = -1; c <= 1; ++c) P3[d][c + 1] = psi_c(c, u[d], u[d] * u[d] + zeta);
+            for (int c = -1; c <= 1; ++c) P3[d][c + 1] = psi_c(c, u[d], fma(u[d], u[d], zeta));
 #pragma unroll
         for (int cz = 0; cz < 3; ++cz)
 #pragma unroll
@@ -959,9 +968,9 @@ __device__ __forceinline__ void ghost_warp(const StepArgs &a, int w)
     }
     // energy set: rho E and H of the state with the ghost's velocity
     const double U = poly5(eu, T), usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    const double rE = rho * (U + 0.5 * usq), P = rho * Rm * T;
+    const double rE = rho * fma(0.5, usq, U), P = rho * Rm * T;
     double q[3], Rt[6], tr3;
-    energy_moments(rho, u, P, U + Rm * T + 0.5 * usq, rE, q, Rt, tr3);
+    energy_moments(rho, u, P, fma(0.5, usq, fma(Rm, T, U)), rE, q, Rt, tr3);
     for (int i = s; i < LBMK_Q; i += S)
         if (live) gh[((size_t)M * LBMK_Q + i) * plane] = grad_dir(i, rE, q, Rt, tr3);
 }
@@ -1141,7 +1150,6 @@ __device__ __forceinline__ double exp_rate(double x)
 #endif
 }
 
-#if !LBMK_FAST
 // exp(x) for x in units of 2^-53 (modulo 2^64) and a float within 1e-4 of it;
 // beyond +-707 from the float alone.
 __device__ __forceinline__ double exp_fixed(long long x, float xf)
@@ -1305,7 +1313,6 @@ __device__ __forceinline__ void molar_production_fixed(const MechConst &mc, doub
         for (int j = 0; j < np; ++j) w.template add<1>(mc.prod[k][j], qt);
     }
 }
-#endif  // !LBMK_FAST
 
 // Molar production rates sum_k (nu''_ak - nu'_ak) q_k at temperature T and
 // concentrations conc, left in sh_w[a * stride + t]; sh_act and sh_g are
@@ -1365,7 +1372,9 @@ __device__ __forceinline__ void molar_production(const MechConst &mc, double T, 
     }
 }
 
-// The rates in sh_w by either form.
+// The rates in sh_w by either form (the fast mixed unit's reported rates keep
+// the hardware exponential; its step takes the integer one, which is both
+// more accurate and faster: k_chem, 160^3, 2.4 ms against 5.4).
 template <int M>
 __device__ __forceinline__ void production_rates(const MechConst &mc, double T, const double *conc, double *sh_act,
                                                  double *sh_g, WReal *sh_w, int t, int stride)
@@ -1397,11 +1406,11 @@ __device__ __forceinline__ double node_temperature(const MechConst &mc, const St
         sh_ra[s * bs] = ra;
     });
     const double u[3] = {sm.j[0] * ir, sm.j[1] * ir, sm.j[2] * ir};
-    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    const double usq = dot3(u, u);
     if (eu_out)
 #pragma unroll
         for (int k = 0; k < 6; ++k) eu_out[k] = eu[k];
-    return solve_T(eu, sm.rhoE * ir - 0.5 * usq, a.macro[(size_t)DR_T * a.N + n], a.status);
+    return solve_T(eu, fma(sm.rhoE, ir, -0.5 * usq), a.macro[(size_t)DR_T * a.N + n], a.status);
 }
 
 // ---------------------------------------------------------------------
@@ -1456,8 +1465,8 @@ __global__ void __launch_bounds__(LBMK_BLOCK, LBMK_MOM_MINB) k_moments(StepArgs 
     });
     const double rho = sm.rho;
     const double u[3] = {sm.j[0] * ir, sm.j[1] * ir, sm.j[2] * ir};
-    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    const double T = solve_T(eu, sm.rhoE * ir - 0.5 * usq, a.macro[DR_T * N + n], a.status);
+    const double usq = dot3(u, u);
+    const double T = solve_T(eu, fma(sm.rhoE, ir, -0.5 * usq), a.macro[DR_T * N + n], a.status);
     const double Rm = mc.r_lat * inv_m;
     if (mask & 2u)
 #pragma unroll
@@ -1542,19 +1551,19 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd, doub
     });
     const double rho = sm.rho, rhoE = sm.rhoE;
     const double u[3] = {sm.j[0] * ir, sm.j[1] * ir, sm.j[2] * ir};
-    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    const double usq = dot3(u, u);
     if (!(rho > 0.0) || !isfinite(rhoE)) flag(a.status, LBMK_BIT_NONFINITE);
     if (neg) flag(a.status, LBMK_BIT_NEGATIVE);
 
     // temperature, Eq. (temperature)
-    const double T = solve_T(eu, rhoE * ir - 0.5 * usq, a.macro[DR_T * N + n], a.status);
+    const double T = solve_T(eu, fma(rhoE, ir, -0.5 * usq), a.macro[DR_T * N + n], a.status);
     const double Rm = mc.r_lat * inv_m;
     const double P = rho * Rm * T;
     // enthalpies, Eq. (specHa); rest-direction equilibria of the species and
     // mixture sets (Eqs. (feq), (feqmix))
     double H = 0.0;
 #if LBMK_MIXED
-    const double c2[3] = {1.0 - u[0] * u[0], 1.0 - u[1] * u[1], 1.0 - u[2] * u[2]};
+    const double c2[3] = {fma(-u[0], u[0], 1.0), fma(-u[1], u[1], 1.0), fma(-u[2], u[2], 1.0)};
 #endif
 #pragma unroll 1
     for (int s = 0; s < M; ++s) {
@@ -1562,7 +1571,7 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd, doub
         H = fma(sh[(M + s) * bs], Ha, H);
         R[(size_t)(rr.h + s) * N + n] = cvt<Real>(Ha);
 #if LBMK_MIXED
-        const double z = (s < M - 1 ? mc.Ra[s] : Rm) * T;
+        const double z = __dmul_rn(s < M - 1 ? mc.Ra[s] : Rm, T);
         const double r = s < M - 1 ? sh[s * bs] : rho;
         a.macro[(size_t)(DR_FEQ0 + s) * N + n] = r * (c2[0] - z) * (c2[1] - z) * (c2[2] - z);
 #endif
@@ -1590,12 +1599,12 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd, doub
     // for the diffusion velocities, added in k_diff; the grad-Y part
     // (Eq. (corrFourier)) needs the neighbours and is added in k_step_g.
     double qeq[3], Rt[6], tr3;
-    energy_moments(rho, u, P, H + 0.5 * usq, rhoE, qeq, Rt, tr3);
-    const double dP[6] = {sm.P[0] - (P + rho * u[0] * u[0]), sm.P[1] - (P + rho * u[1] * u[1]),
-                          sm.P[2] - (P + rho * u[2] * u[2]), sm.P[3] - rho * u[0] * u[1],
-                          sm.P[4] - rho * u[0] * u[2], sm.P[5] - rho * u[1] * u[2]};
-    const double uP[3] = {u[0] * dP[0] + u[1] * dP[3] + u[2] * dP[4], u[0] * dP[3] + u[1] * dP[1] + u[2] * dP[5],
-                          u[0] * dP[4] + u[1] * dP[5] + u[2] * dP[2]};
+    energy_moments(rho, u, P, fma(0.5, usq, H), rhoE, qeq, Rt, tr3);
+    const double ru[3] = {rho * u[0], rho * u[1], rho * u[2]};
+    const double dP[6] = {sm.P[0] - fma(ru[0], u[0], P), sm.P[1] - fma(ru[1], u[1], P), sm.P[2] - fma(ru[2], u[2], P),
+                          fma(-ru[0], u[1], sm.P[3]),    fma(-ru[0], u[2], sm.P[4]),    fma(-ru[1], u[2], sm.P[5])};
+    const double row0[3] = {dP[0], dP[3], dP[4]}, row1[3] = {dP[3], dP[1], dP[5]}, row2[3] = {dP[4], dP[5], dP[2]};
+    const double uP[3] = {dot3(u, row0), dot3(u, row1), dot3(u, row2)};
 
     // the record: double rows
     a.macro[DR_T * N + n] = T;
@@ -1613,11 +1622,11 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd, doub
     // storage-type rows
     R[(size_t)rr.nup * N + n] = nup;
     // Phi (Eq. (Xalpha)), stored in the storage type and formed in it
-    const Real rhoR = cvt<Real>(rho), rtR = cvt<Real>(Rm * T), ph = (Real)1 - (Real)3 * rtR;
+    const Real rhoR = cvt<Real>(rho), rtR = cvt<Real>(Rm * T), ph = fma((Real)-3, rtR, (Real)1);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         const Real ud = cvt<Real>(u[d]);
-        R[(size_t)(rr.phi + d) * N + n] = rhoR * ud * (ph - ud * ud);
+        R[(size_t)(rr.phi + d) * N + n] = rhoR * ud * fma(-ud, ud, ph);
         R[(size_t)(rr.u + d) * N + n] = ud;
         // the difference is formed in double (it cancels), the product in the storage type
         R[(size_t)(rr.dq + d) * N + n] = (omega - omega1) * cvt<Real>(sm.q[d] - uP[d] - qeq[d]);
@@ -1825,6 +1834,75 @@ __global__ void __launch_bounds__(LBMK_BLOCK, LBMK_DIFF_MINB) k_diff(StepArgs a)
 }
 
 // ---------------------------------------------------------------------
+// Pass 1c: production rates rho_dot_a of the record's state, in the storage
+// type, into the rows that held rho_a for the diffusion pass.  A kernel of
+// its own: inside the collision its double operations, a serial chain of 64
+// cycles each, ran at the collision's 8 to 12 warps per SM and barely
+// overlapped it (256^3 mixed: 25.2 ms in one kernel, 9.9 + 12.1 ms in two;
+// 128^3 double: 11.1 ms, 1.4 + 8.0 ms).  64 registers, 256-thread blocks at 4
+// per SM: 9.9 ms; 3 per SM 10.0, 2 per SM 10.3.
+// sh: shared memory, chem_cols<M>() columns of bs doubles.
+// ---------------------------------------------------------------------
+template <int M>
+constexpr int chem_cols() { return 3 * M; }
+
+__device__ __forceinline__ Real *rate_rows(const StepArgs &a, int M, Real *R)
+{
+#if LBMK_MIXED
+    (void)R;
+    return reinterpret_cast<Real *>(a.macro + (size_t)dr_ra(M) * a.N);
+#else
+    return R + (size_t)rec_rows(M, false).ra * a.N;
+#endif
+}
+
+template <int M>
+__device__ __forceinline__ void chem_node(const StepArgs &a, int n, double *sh, int bs)
+{
+    const MechConst &mc = c_mech[a.slot];
+    const int t = threadIdx.x;
+    const size_t N = a.N;
+    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    Real *R = rec(a);
+    const double T = a.macro[(size_t)DR_T * N + n];
+    const Real rho = R[(size_t)rr.rho * N + n];
+    double *sh_act = sh, *sh_g = sh + M * bs;
+    WReal *sh_w = reinterpret_cast<WReal *>(sh + 2 * M * bs);
+    double conc[M];
+#pragma unroll
+    for (int s = 0; s < M; ++s) {
+#if LBMK_MIXED
+        conc[s] = cvt<double>(rho) * cvt<double>(R[(size_t)(rr.y + s) * N + n]) * mc.invW[s];
+#else
+        conc[s] = rho * R[(size_t)(rr.y + s) * N + n] * mc.invW[s];
+#endif
+    }
+    Real *wd = rate_rows(a, M, R) + n;
+#if LBMK_MIXED
+    if (mc.chem_fixed) {
+        const RateSums<true> w{sh + 2 * M * bs + t, bs};
+        molar_production_fixed<M, true>(mc, T, conc, sh_act, sh_g, w, t, bs);
+#pragma unroll
+        for (int s = 0; s < M; ++s) wd[(size_t)s * N] = w.mass_float(s, mc.W[s]);
+        return;
+    }
+#endif
+    production_rates<M>(mc, T, conc, sh_act, sh_g, sh_w, t, bs);
+#pragma unroll
+    for (int s = 0; s < M; ++s) wd[(size_t)s * N] = cvt<Real>(mc.W[s] * sh_w[s * bs + t]);
+}
+
+extern __shared__ double sh_chem[];
+
+template <int M>
+__global__ void __launch_bounds__(LBMK_MAXBLOCK, LBMK_CHEM_MINB) k_chem(StepArgs a)
+{
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= a.N) return;
+    chem_node<M>(a, n, sh_chem, blockDim.x);
+}
+
+// ---------------------------------------------------------------------
 // Pass 2: G_alpha = (1/omega - 1/2) d_alpha Phi_alpha with the isotropic
 // gradient d_alpha phi = (1/theta) sum_i w_i c_ia phi(x + c_i).
 // ---------------------------------------------------------------------
@@ -1969,13 +2047,13 @@ __global__ void __launch_bounds__(LBMK_MAXBLOCK) k_step_g(StepArgs a)
 // ---------------------------------------------------------------------
 #if LBMK_MIXED
 template <int M>
-constexpr int step_cols() { return 3 * M; }      // scratch columns of the production rates
+constexpr int step_cols() { return 0; }
 
 template <int M, bool FX>
 __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, double *sh, int bs)
 {
-    double *sh_act = sh, *sh_g = sh + M * bs;
-    WReal *sh_w = reinterpret_cast<WReal *>(sh + 2 * M * bs);
+    (void)sh;
+    (void)bs;
     const MechConst &mc = c_mech[a.slot];
     const int n = nd.n;
     const size_t N = a.N;
@@ -2019,25 +2097,7 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
 #pragma unroll
         for (int d = 0; d < 3; ++d) xs[s][d] = u[d] + ld(rr.du + 3 * s + d);
         bt[s] = ld(rr.beta + s);
-    }
-    {
-        // the production rates of this node
-        double conc[M];
-#pragma unroll
-        for (int s = 0; s < M; ++s) conc[s] = cvt<double>(rho) * cvt<double>(Yl[s]) * mc.invW[s];
-#if !LBMK_FAST
-        if (mc.chem_fixed) {
-            const RateSums<true> w{sh_w + threadIdx.x, bs};
-            molar_production_fixed<M, true>(mc, ldd(DR_T), conc, sh_act, sh_g, w, threadIdx.x, bs);
-#pragma unroll
-            for (int s = 0; s < M; ++s) wd[s] = w.mass_float(s, mc.W[s]);
-        } else
-#endif
-        {
-            molar_production<M>(mc, ldd(DR_T), conc, sh_act, sh_g, sh_w, threadIdx.x, bs);
-#pragma unroll
-            for (int s = 0; s < M; ++s) wd[s] = cvt<Real>(mc.W[s] * sh_w[s * bs + threadIdx.x]);
-        }
+        wd[s] = rate_rows(a, M, rec(a))[(size_t)s * N + n];
     }
     const Real u2[3] = {u[0] * u[0], u[1] * u[1], u[2] * u[2]};
 
@@ -2178,9 +2238,15 @@ namespace {
 template <int M>
 constexpr bool kFixedStep = M >= 4 && !LBMK_MIXED;
 
-// Shared memory of a block of bs threads for step_node.
+// Shared memory of a block of bs threads for step_node, and for all phases of
+// the persistent kernel.
 template <int M>
 constexpr size_t step_smem(int bs) { return (size_t)step_cols<M>() * bs * sizeof(double); }
+template <int M>
+constexpr size_t persist_smem(int bs)
+{
+    return (size_t)(step_cols<M>() > chem_cols<M>() ? step_cols<M>() : chem_cols<M>()) * bs * sizeof(double);
+}
 
 extern __shared__ double sh_step[];
 
@@ -2258,7 +2324,13 @@ int launch_one(const StepArgs &a, int k)
             k_diff<M, false><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a);
         break;
     }
-    case LBMK_K_CHEM: break;            // the rates are formed inside k_step
+    case LBMK_K_CHEM: {
+        static std::atomic<unsigned long long> opted{0};
+        const int e = opt_in_smem(k_chem<M>, chem_cols<M>() * LBMK_MAXBLOCK * sizeof(double), opted);
+        if (e) return e;
+        k_chem<M><<<grid_for(a.N, bs), bs, chem_cols<M>() * bs * sizeof(double), a.stream>>>(a);
+        break;
+    }
     case LBMK_K_GRAD: k_grad<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
     case LBMK_K_STEPG: k_step_g<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
     case LBMK_K_STEP: {
@@ -2361,7 +2433,10 @@ __device__ __forceinline__ bool persist_step(const StepArgs &b, int tile, GridBa
     // each one's arithmetic as in its own kernel (no values shared)
     tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) { collide_energy<M>(b, nd); });
     if (!grid_barrier(bar, nb, cap, b.status)) return false;
-    tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) { step_node<M, FX && kFixedStep<M>>(b, nd, sh_step, LBMK_BLOCK); });
+    tile_loop<M>(b, tile, &bar->next, [&](const Node &nd) {
+        chem_node<M>(b, nd.n, sh_step, LBMK_BLOCK);
+        step_node<M, FX && kFixedStep<M>>(b, nd, sh_step, LBMK_BLOCK);
+    });
     return grid_barrier(bar, nb, cap, b.status);
 }
 
@@ -2385,10 +2460,10 @@ int launch_persistent(const StepArgs &a, int nsteps, int tile_mult, GridBarrier 
     if (nsteps < 1 || tile_mult < 1) return (int)cudaErrorInvalidValue;
     int per_sm = 0, dev = 0, nsm = 0;
     static std::atomic<unsigned long long> opted{0};
-    const int eo = opt_in_smem(k_persist<M, FX>, step_smem<M>(LBMK_BLOCK), opted);
+    const int eo = opt_in_smem(k_persist<M, FX>, persist_smem<M>(LBMK_BLOCK), opted);
     if (eo) return eo;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_persist<M, FX>, LBMK_BLOCK,
-                                                                  step_smem<M>(LBMK_BLOCK));
+                                                                  persist_smem<M>(LBMK_BLOCK));
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return (int)e;
@@ -2404,7 +2479,7 @@ int launch_persistent(const StepArgs &a, int nsteps, int tile_mult, GridBarrier 
     unsigned cc = cap;
     void *args[] = {(void *)&a0, (void *)&a1, (void *)&ns, (void *)&tl, (void *)&bb, (void *)&cc};
     return (int)cudaLaunchCooperativeKernel((const void *)k_persist<M, FX>, dim3(blocks), dim3(LBMK_BLOCK), args,
-                                            step_smem<M>(LBMK_BLOCK), a.stream);
+                                            persist_smem<M>(LBMK_BLOCK), a.stream);
 }
 template <int M>
 int run_persistent(const StepArgs &a, int nsteps, int tile_mult, GridBarrier *bar, unsigned cap)
