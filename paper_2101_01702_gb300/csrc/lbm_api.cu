@@ -1048,7 +1048,9 @@ int lbm_flame_speeds(lbm_ctx *c, double *Sd, double *Sa)
     // point of the next step): kept aside and put back
     int st = copy_d2d(tkeep, Trow, N * sizeof(double), c->stream);
     if (st != LBM_OK) return st;
-    if (ops(c->lat.precision).flame(args_of(c), scr, dSd, dSa)) return LBM_ERR_CUDA;
+    StepArgs a = args_of(c);
+    a.dst = scr;                   // the record pass's own scratch (DiffRows), done with before scr is written
+    if (ops(c->lat.precision).flame(a, scr, dSd, dSa)) return LBM_ERR_CUDA;
     if (!dev) {
         st = check_cuda(cudaMemcpyAsync(Sd, dSd, N * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         if (st == LBM_OK) st = check_cuda(cudaMemcpyAsync(Sa, dSa, N * sizeof(double), cudaMemcpyDeviceToHost, c->stream));

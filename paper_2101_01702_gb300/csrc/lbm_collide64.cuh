@@ -49,7 +49,7 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
     const MechConst &mc = c_mech[a.slot];
     const int n = nd.n, t = threadIdx.x;
     const size_t N = a.N;
-    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    const RecRows rr = rec_rows(M);
     const double *R = rec(a);
     auto ld = [&](int row) { return R[(size_t)row * N + n]; };
 
@@ -58,7 +58,7 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
     double Rw[M], kf[M - 1], kE[M - 1], kF[M - 1];
     {
         const double kappa = ld(rr.kappa);
-        const double *wd = rate_rows(a, M, rec(a)) + n;
+        const double *wd = R + (size_t)rr.wd * N + n;
 #pragma unroll
         for (int s = 0; s < M; ++s) {
             const double Y = ld(rr.y + s), ra = rho * Y, wscale = FX ? mc.invW[s] : 1.0;

@@ -36,40 +36,42 @@ struct GridBarrier {
 //   DR_FEQ0   rest-direction equilibrium of the species and mixture sets (M)
 //   DR_GE     rho E            DR_GQ  q^eq (3)       DR_GR  R^eq - rho E theta I (6: xx yy zz xy xz yz)
 //   DR_GTR    tr(R^eq - rho E theta I) / 3
-//   in mixed precision also DR_RA rho_a (M), DR_U u (3), DR_HK kappa/(2 rho)
-//   (fast mixed: 1/rho): what the diffusion pass (k_diff) needs in double
 // Storage-type rows:
 //   nup  1/omega - 1/2      phi  Phi (3)        g    G (3)
 //   y    Y_a (M)            rho  rho            u    u (3)
 //   du   du_a (3M, a-major; until k_diff the momenta j_a)   beta beta_a (M)
-//   ra   rho_a (M; double precision only)
+//   wd   rho_dot_a (M; double precision: rho_a until k_chem)
 //   kappa m R_U T           rt   R T            om   omega      om1 omega_1
 //   p    P                  dq   (omega - omega_1)(q* - q^eq) without the grad-Y part (3; until k_diff
 //                                also without the part of the diffusion velocities)
 //   h    H_a (M)
+// What k_diff needs in double of a mixed state waits in the buffer that the
+// step writes, unused until the collisions (DiffRows): rows of doubles at its
+// start, fewer bytes than the float populations for every M.
 #define DR_T 0
 #define DR_FEQ0 1
 __host__ __device__ constexpr int dr_ge(int M) { return M + 1; }
 __host__ __device__ constexpr int dr_gq(int M) { return M + 2; }
 __host__ __device__ constexpr int dr_gr(int M) { return M + 5; }
 __host__ __device__ constexpr int dr_gtr(int M) { return M + 11; }
-__host__ __device__ constexpr int dr_ra(int M) { return M + 12; }
-__host__ __device__ constexpr int dr_u(int M) { return 2 * M + 12; }
-__host__ __device__ constexpr int dr_hk(int M) { return 2 * M + 15; }
-__host__ __device__ constexpr int macro_double_rows(int M, bool mixed) { return mixed ? 2 * M + 16 : M + 12; }
-struct RecRows {
-    int nup, phi, g, y, rho, u, du, beta, kappa, rt, om, om1, p, dq, h, ra, total;
+__host__ __device__ constexpr int macro_double_rows(int M) { return M + 12; }
+// rho_a (M), u (3), kappa/(2 rho) (fast mixed: 1/rho)
+struct DiffRows {
+    int ra, u, hk, total;
 };
-__host__ __device__ constexpr RecRows rec_rows(int M, bool mixed)
+__host__ __device__ constexpr DiffRows diff_rows(int M) { return DiffRows{0, M, M + 3, M + 4}; }
+struct RecRows {
+    int nup, phi, g, y, rho, u, du, beta, kappa, rt, om, om1, p, dq, h, wd, total;
+};
+__host__ __device__ constexpr RecRows rec_rows(int M)
 {
     return RecRows{0, 1, 4, 7, 7 + M, 8 + M, 11 + M, 11 + 4 * M, 11 + 5 * M, 12 + 5 * M, 13 + 5 * M,
-                   14 + 5 * M, 15 + 5 * M, 16 + 5 * M, 19 + 5 * M, 19 + 6 * M, 19 + (mixed ? 6 : 7) * M};
+                   14 + 5 * M, 15 + 5 * M, 16 + 5 * M, 19 + 5 * M, 19 + 6 * M, 19 + 7 * M};
 }
 // Bytes of the macro buffer for N nodes, M species and a storage element size.
 __host__ __device__ constexpr size_t macro_bytes_for(int M, size_t N, size_t real_size)
 {
-    const bool mixed = real_size == sizeof(float);
-    return (size_t)macro_double_rows(M, mixed) * N * sizeof(double) + (size_t)rec_rows(M, mixed).total * N * real_size;
+    return (size_t)macro_double_rows(M) * N * sizeof(double) + (size_t)rec_rows(M).total * N * real_size;
 }
 
 // Population buffer.
@@ -220,8 +222,9 @@ int init_fp64(const StepArgs &a, const double *X, const double *T, const double 
 int init_mixed(const StepArgs &a, const double *X, const double *T, const double *u, double P);
 int init_mixed_fast(const StepArgs &a, const double *X, const double *T, const double *u, double P);
 
-// one full time step src -> dst (ghost, moments, production rates,
-// gradients, energy collision, species/mixture collision); with ev !=
+// one full time step src -> dst (ghost, moments with the diffusion
+// velocities, production rates, gradients, energy collision,
+// species/mixture collision); with ev !=
 // nullptr, events ev[0..6] are recorded around the six phases
 int step_fp64(const StepArgs &a, cudaEvent_t *ev = nullptr);
 int step_mixed(const StepArgs &a, cudaEvent_t *ev = nullptr);

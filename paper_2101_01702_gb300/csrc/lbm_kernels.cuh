@@ -440,7 +440,7 @@ __device__ __forceinline__ size_t nb_of(const StencilIdx &t, const StepArgs &a)
 
 __device__ __forceinline__ Real *rec(const StepArgs &a)
 {
-    return reinterpret_cast<Real *>(a.macro + (size_t)macro_double_rows(a.M, LBMK_MIXED) * a.N);
+    return reinterpret_cast<Real *>(a.macro + (size_t)macro_double_rows(a.M) * a.N);
 }
 
 // ---------------------------------------------------------------------
@@ -1519,10 +1519,13 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd, doub
     const MechConst &mc = c_mech[a.slot];
     const int n = nd.n;
     const size_t N = a.N;
-    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    const RecRows rr = rec_rows(M);
     Real *R = rec(a);
     PullIdx p;
     make_pull(p, nd, a);
+#if LBMK_MIXED
+    double *dr = static_cast<double *>(a.dst) + n;          // DiffRows
+#endif
     Sums sm = {};
     double ir = 0.0, inv_m = 0.0, eu[6];
     bool neg = false;
@@ -1544,9 +1547,9 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd, doub
         sh[(M + s) * bs] = Y;
         R[(size_t)(rr.y + s) * N + n] = cvt<Real>(Y);
 #if LBMK_MIXED
-        a.macro[(size_t)(dr_ra(M) + s) * N + n] = ra;
+        dr[(size_t)(diff_rows(M).ra + s) * N] = ra;
 #else
-        R[(size_t)(rr.ra + s) * N + n] = ra;
+        R[(size_t)(rr.wd + s) * N + n] = ra;
 #endif
     });
     const double rho = sm.rho, rhoE = sm.rhoE;
@@ -1616,8 +1619,8 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd, doub
     a.macro[(size_t)dr_gtr(M) * N + n] = tr3;
 #if LBMK_MIXED
 #pragma unroll
-    for (int d = 0; d < 3; ++d) a.macro[(size_t)(dr_u(M) + d) * N + n] = u[d];
-    a.macro[(size_t)dr_hk(M) * N + n] = LBMK_FAST ? ir : 0.5 * kappa * ir;
+    for (int d = 0; d < 3; ++d) dr[(size_t)(diff_rows(M).u + d) * N] = u[d];
+    dr[(size_t)diff_rows(M).hk * N] = LBMK_FAST ? ir : 0.5 * kappa * ir;
 #endif
     // storage-type rows
     R[(size_t)rr.nup * N + n] = nup;
@@ -1673,15 +1676,18 @@ __device__ __forceinline__ void diff_node(const StepArgs &a, const Node &nd, dou
     const MechConst &mc = c_mech[a.slot];
     const int n = nd.n;
     const size_t N = a.N;
-    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    const RecRows rr = rec_rows(M);
     Real *R = rec(a);
     auto ld = [&](int row) { return R[(size_t)row * N + n]; };
     Real duR[M][3], itaR[M];
+#if LBMK_MIXED
+    const double *dr = static_cast<const double *>(a.dst) + n;
+#endif
 #if LBMK_MIXED && !LBMK_FAST
     if constexpr (kRefined<M, FX>) {
         bool bad = false;
-        diffusion_refined<M>(mc, a.macro + (size_t)dr_ra(M) * N + n, a.macro + (size_t)dr_u(M) * N + n,
-                             R + (size_t)rr.du * N + n, N, a.macro[(size_t)dr_hk(M) * N + n], sh, bs, duR, itaR, &bad);
+        diffusion_refined<M>(mc, dr + (size_t)diff_rows(M).ra * N, dr + (size_t)diff_rows(M).u * N,
+                             R + (size_t)rr.du * N + n, N, dr[(size_t)diff_rows(M).hk * N], sh, bs, duR, itaR, &bad);
         if (bad) flag(a.status, LBMK_BIT_PIVOT);
     } else
 #endif
@@ -1693,16 +1699,16 @@ __device__ __forceinline__ void diff_node(const StepArgs &a, const Node &nd, dou
     Real ja[M][3];
     {
 #if LBMK_MIXED
-        const double *ra = a.macro + (size_t)dr_ra(M) * N + n;
+        const double *ra = dr + (size_t)diff_rows(M).ra * N;
 #pragma unroll
-        for (int d = 0; d < 3; ++d) ur[d] = cvt<SReal>(a.macro[(size_t)(dr_u(M) + d) * N + n]);
+        for (int d = 0; d < 3; ++d) ur[d] = cvt<SReal>(dr[(size_t)(diff_rows(M).u + d) * N]);
 #else
-        const double *ra = R + (size_t)rr.ra * N + n;
+        const double *ra = R + (size_t)rr.wd * N + n;
 #pragma unroll
         for (int d = 0; d < 3; ++d) ur[d] = ld(rr.u + d);
 #endif
 #if LBMK_FAST
-        irr = cvt<SReal>(a.macro[(size_t)dr_hk(M) * N + n]);
+        irr = cvt<SReal>(dr[(size_t)diff_rows(M).hk * N]);
         kap = ld(rr.kappa);
 #pragma unroll
         for (int s = 0; s < M; ++s) Yr[s] = ld(rr.y + s);
@@ -1713,7 +1719,7 @@ __device__ __forceinline__ void diff_node(const StepArgs &a, const Node &nd, dou
         for (int s = 0; s < M; ++s) rho += ra[(size_t)s * N];
         irr = 1.0 / rho;
 #if LBMK_MIXED
-        kap = 2.0 * a.macro[(size_t)dr_hk(M) * N + n] * rho;
+        kap = 2.0 * dr[(size_t)diff_rows(M).hk * N] * rho;
 #else
         kap = ld(rr.kappa);
 #endif
@@ -1835,7 +1841,7 @@ __global__ void __launch_bounds__(LBMK_BLOCK, LBMK_DIFF_MINB) k_diff(StepArgs a)
 
 // ---------------------------------------------------------------------
 // Pass 1c: production rates rho_dot_a of the record's state, in the storage
-// type, into the rows that held rho_a for the diffusion pass.  A kernel of
+// type (in double, into the rows that held rho_a for k_diff).  A kernel of
 // its own: inside the collision its double operations, a serial chain of 64
 // cycles each, ran at the collision's 8 to 12 warps per SM and barely
 // overlapped it (256^3 mixed: 25.2 ms in one kernel, 9.9 + 12.1 ms in two;
@@ -1846,23 +1852,13 @@ __global__ void __launch_bounds__(LBMK_BLOCK, LBMK_DIFF_MINB) k_diff(StepArgs a)
 template <int M>
 constexpr int chem_cols() { return 3 * M; }
 
-__device__ __forceinline__ Real *rate_rows(const StepArgs &a, int M, Real *R)
-{
-#if LBMK_MIXED
-    (void)R;
-    return reinterpret_cast<Real *>(a.macro + (size_t)dr_ra(M) * a.N);
-#else
-    return R + (size_t)rec_rows(M, false).ra * a.N;
-#endif
-}
-
 template <int M>
 __device__ __forceinline__ void chem_node(const StepArgs &a, int n, double *sh, int bs)
 {
     const MechConst &mc = c_mech[a.slot];
     const int t = threadIdx.x;
     const size_t N = a.N;
-    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    const RecRows rr = rec_rows(M);
     Real *R = rec(a);
     const double T = a.macro[(size_t)DR_T * N + n];
     const Real rho = R[(size_t)rr.rho * N + n];
@@ -1877,7 +1873,7 @@ __device__ __forceinline__ void chem_node(const StepArgs &a, int n, double *sh, 
         conc[s] = rho * R[(size_t)(rr.y + s) * N + n] * mc.invW[s];
 #endif
     }
-    Real *wd = rate_rows(a, M, R) + n;
+    Real *wd = R + (size_t)rr.wd * N + n;
 #if LBMK_MIXED
     if (mc.chem_fixed) {
         const RateSums<true> w{sh + 2 * M * bs + t, bs};
@@ -1910,7 +1906,7 @@ template <int M>
 __device__ __forceinline__ void grad_node(const StepArgs &a, const Node &nd)
 {
     const size_t N = a.N;
-    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    const RecRows rr = rec_rows(M);
     Real *R = rec(a);
     const Real *Phi = R + (size_t)rr.phi * N;
     StencilIdx st;
@@ -1953,7 +1949,7 @@ __device__ __forceinline__ void collide_energy(const StepArgs &a, const Node &nd
 {
     const int n = nd.n;
     const size_t N = a.N;
-    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    const RecRows rr = rec_rows(M);
     const Real *R = rec(a);
     auto ld = [&](int row) { return R[(size_t)row * N + n]; };
     auto ldd = [&](int row) { return a.macro[(size_t)row * N + n]; };
@@ -2057,7 +2053,7 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
     const MechConst &mc = c_mech[a.slot];
     const int n = nd.n;
     const size_t N = a.N;
-    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    const RecRows rr = rec_rows(M);
     const Real *R = rec(a);
     auto ld = [&](int row) { return R[(size_t)row * N + n]; };
     auto ldd = [&](int row) { return a.macro[(size_t)row * N + n]; };
@@ -2097,7 +2093,7 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
 #pragma unroll
         for (int d = 0; d < 3; ++d) xs[s][d] = u[d] + ld(rr.du + 3 * s + d);
         bt[s] = ld(rr.beta + s);
-        wd[s] = rate_rows(a, M, rec(a))[(size_t)s * N + n];
+        wd[s] = ld(rr.wd + s);
     }
     const Real u2[3] = {u[0] * u[0], u[1] * u[1], u[2] * u[2]};
 
@@ -3020,7 +3016,7 @@ __global__ void __launch_bounds__(LBMK_BLOCK) k_flame1(StepArgs a, double *scr)
     if (!node_of(nd, a)) return;
     const size_t N = a.N;
     const int n = nd.n;
-    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    const RecRows rr = rec_rows(M);
     const Real *R = rec(a);
     const double *Tr = a.macro + (size_t)DR_T * N;
     StencilIdx st;
@@ -3055,7 +3051,7 @@ __global__ void __launch_bounds__(LBMK_HRR_THREADS) k_flame2(StepArgs a, const d
     if (!node_of(nd, a)) return;
     const size_t N = a.N;
     const int n = nd.n;
-    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    const RecRows rr = rec_rows(M);
     const Real *R = rec(a);
     StencilIdx st;
     make_stencil(st, nd, a);
