@@ -443,7 +443,7 @@ __device__ void adj_collide_node(const MechConst &mc, const StepArgs &a, const A
 #pragma unroll
     for (int s = 0; s < M; ++s) gY[s][0] = gY[s][1] = gY[s][2] = 0.0;
     {
-        const RecRows rr = rec_rows(M, LBMK_MIXED);
+        const RecRows rr = rec_rows(M);
         const double *Rr = rec(a);
         StencilIdx st;
         make_stencil(st, nd, a);
@@ -852,7 +852,7 @@ __global__ void __launch_bounds__(LBMK_BLOCK) k_adj_grad1(StepArgs a, AdjBufs g)
     Node nd;
     if (!node_of(nd, a)) return;
     const size_t N = a.N;
-    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    const RecRows rr = rec_rows(M);
     const double *Rr = rec(a);
     StencilIdx st;
     make_stencil(st, nd, a);
@@ -898,7 +898,7 @@ __global__ void __launch_bounds__(LBMK_BLOCK) k_adj_finish(StepArgs a, AdjBufs g
     if (!node_of(nd, a)) return;
     const size_t N = a.N;
     const int n = nd.n;
-    const RecRows rr = rec_rows(M, LBMK_MIXED);
+    const RecRows rr = rec_rows(M);
     const double *Rr = rec(a);
     StencilIdx st;
     make_stencil(st, nd, a);
