@@ -225,8 +225,9 @@ int lbm_step_graph(lbm_ctx *ctx, int n);
 /* n time steps in ONE persistent, cooperative kernel launch (the paper has
  * no counterpart: a launch structure for batches of small lattices, such as
  * the quasi-1D flames of Sec. 5a side by side).  The blocks stay resident;
- * in each phase of a step (ghost planes, the per-node record, G, the
- * energy collision, the species collision) their warps take chunks of
+ * in each phase of a step (ghost planes, the per-node record with the
+ * diffusion velocities, G, the energy collision, the production rates with
+ * the species collision) their warps take chunks of
  * tile_mult x 32 consecutive nodes from a queue, and all meet at a grid
  * barrier before the next phase.  Results agree with lbm_step to rounding
  * (the compiler may fuse a multiply and an add in this kernel where it does
@@ -237,9 +238,8 @@ int lbm_step_graph(lbm_ctx *ctx, int n);
  * so the launch always ends -- the state is then partly stepped and must be
  * re-initialised or restored.  tile_mult >= 1.  Waits for the stream and
  * returns like lbm_sync (LBM_ERR_BARRIER after a timeout); LBM_ERR_ARG for
- * n < 0 or tile_mult < 1; LBM_ERR_UNSUPPORTED in a build whose production
- * rates run in a kernel of their own (LBMK_FUSE_CHEM=0); LBM_ERR_CUDA when
- * the device cannot hold the grid's blocks at once. */
+ * n < 0 or tile_mult < 1; LBM_ERR_CUDA when the device cannot hold the
+ * grid's blocks at once. */
 int lbm_step_persistent(lbm_ctx *ctx, int n, int tile_mult, unsigned spin_cap);
 
 /* Picks the tile length of lbm_step_persistent (tile_mult in 1, 2, 4, 8)
@@ -261,9 +261,10 @@ int lbm_autotune_persistent(lbm_ctx *ctx, int steps, int *tile_mult_out);
  * are bit for bit those of the untuned context.  Allocates and frees one
  * temporary row of N doubles.  block_out (NULL or 6 ints) receives the
  * chosen blocks in launch order: ghost nodes, moments, production rates,
- * gradients, energy collision, species/mixture collision (the production-
- * rate entry has no effect: the rates are formed inside the species
- * collision).  Waits for the stream; returns like lbm_sync. */
+ * gradients, energy collision, species/mixture collision (the moment entry
+ * covers the diffusion-velocity kernel as well).  A context that is not
+ * tuned takes blocks by the lattice's size.  Waits for the stream; returns
+ * like lbm_sync. */
 int lbm_autotune(lbm_ctx *ctx, int trials, int *block_out);
 
 /* Sets the block sizes of the six kernels directly (for instance a choice
@@ -279,9 +280,9 @@ int lbm_set_blocks(lbm_ctx *ctx, const int *blocks);
  * the summed device time of the ghost-node, moment, production-rate,
  * gradient, energy-collision and species/mixture-collision kernels over
  * the n steps, phase_ms[LBM_PHASES] the device time from the first launch
- * to the end of the last.  The production rates are formed inside the
- * species/mixture-collision kernel (no kernel of their own), so their phase
- * is empty and their time is in phase_ms[5].  Returns like lbm_step. */
+ * to the end of the last.  The diffusion velocities, a kernel between the
+ * moments and the production rates, are counted with the moments.  Returns
+ * like lbm_step. */
 #define LBM_PHASES 6
 int lbm_step_timed(lbm_ctx *ctx, int n, double *phase_ms);
 

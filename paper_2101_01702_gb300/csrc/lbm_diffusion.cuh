@@ -19,7 +19,7 @@
 // pairs of floats), 2^-45 of their largest term; the correction, solved with the same
 // factors, is then good to 2^-40 of x, and x0 plus it is rounded to float
 // once -- the float that the double solution rounds to, but for ties
-// (tests/test_gpu_diffusion.py measures both against 64-bit solutions).
+// (tests/test_diffusion_host.py measures both against a 128-bit solution).
 //
 // A double LDL^T solve costs 740 FP64 instructions per warp at nine species,
 // 56 thousand cycles of a scheduler; this one about 7 thousand
