@@ -39,24 +39,24 @@ FP64_PEAK_TFLOPS_DERIVED = SM_COUNT * FP64_FMA_PER_SM_CLK * 2 * SM_MAX_MHZ * 1e6
 
 # Per lattice node and launch, counted by ncu for the kernels as they
 # stand (profiles/ has the captures and their commands):
-#   FP64 flops = 2 x DFMA + DADD + DMUL thread instructions (64^3 instance:
-#   instruction counts per node do not depend on the lattice size);
-#   DRAM bytes = dram__bytes_read.sum + dram__bytes_write.sum on the 256^3
-#   lattice itself (a smaller one keeps part of its state in L2).
-# The production rates are formed inside k_step (no k_chem launch), so
-# their flops count there.
+#   FP64 flops = 2 x DFMA + DADD + DMUL thread instructions, and DRAM bytes =
+#   dram__bytes_read.sum + dram__bytes_write.sum, of the 96^3 instance (0.9 M
+#   nodes, a state of 1.1 GB, nine times the L2).
+# "k_pre" is the moment phase: k_pre and k_diff (diffusion velocities)
+# together.  In the mixed unit k_diff and the sums of k_pre and k_chem that
+# run on the integer and float pipes count no FP64 flops.
 FP64_FLOPS_PER_NODE = {
-    "mixed": {"k_pre": 1873.6, "k_step_g": 165.0, "k_step": 1189.0},
-    "mixed_fast": {"k_pre": 621.5, "k_step_g": 165.0, "k_step": 663.0},
-    "fp64": {"k_pre": 2561.6, "k_step_g": 737.0, "k_step": 13688.0},
+    "mixed": {"k_pre": 514.1, "k_chem": 333.0, "k_step_g": 165.0, "k_step": 18.0},
+    "mixed_fast": {"k_pre": 503.1, "k_chem": 333.0, "k_step_g": 165.0, "k_step": 18.0},
+    "fp64": {"k_pre": 1932.1, "k_chem": 420.0, "k_step_g": 737.0, "k_step": 2636.0},
 }
 # lbm_heat_release (k_hrr: moments, temperature, hdot^c and its derivatives
 # per node), counted the same way; None until counted.
-HRR_FLOPS_PER_NODE = {"mixed": 3123.0, "mixed_fast": None, "fp64": None}
+HRR_FLOPS_PER_NODE = {"mixed": 2147.0, "mixed_fast": None, "fp64": None}
 DRAM_BYTES_PER_NODE = {
-    "mixed": {"k_pre": 2165.2, "k_step_g": 617.3, "k_step": 2438.2},
-    "mixed_fast": {"k_pre": 2275.2, "k_step_g": 600.5, "k_step": 2398.0},
-    "fp64": {"k_pre": 3415.9, "k_step_g": 699.7, "k_step": 4458.0},
+    "mixed": {"k_pre": 2720.2, "k_chem": 53.6, "k_step_g": 577.6, "k_step": 2388.4},
+    "mixed_fast": {"k_pre": 2648.8, "k_chem": 53.3, "k_step_g": 577.8, "k_step": 2388.3},
+    "fp64": {"k_pre": 4461.6, "k_chem": 118.5, "k_step_g": 680.6, "k_step": 4489.4},
 }
 
 
@@ -551,8 +551,8 @@ def run_ours(args):
         fast = {"mlups": N * args.steps * world / (msf * 1e-3) / 1e6, "steps": args.steps,
                 "phase_ms": {"moments": phf[1], "chemistry": phf[2], "gradients": phf[3],
                              "energy_collision": phf[4], "species_collision": phf[5]},
-                "note": "LBM_MIXED_FAST: Stefan-Maxwell solve and relaxation in float, exponentials of the "
-                        "rates with a float 2^f; same storage and accuracy bar"}
+                "note": "LBM_MIXED_FAST: Stefan-Maxwell solve and relaxation in float; same storage and "
+                        "accuracy bar"}
         sf.close()
         del sf
         torch.cuda.empty_cache()
@@ -573,7 +573,7 @@ def run_ours(args):
         mst = float(pht[lbm.LBM_PHASES])
         pht = pht[:lbm.LBM_PHASES] / args.steps
         transport = {"mlups": N * args.steps * world / (mst * 1e-3) / 1e6, "steps": args.steps,
-                     "phase_ms": {"moments": pht[1], "gradients": pht[3], "energy_collision": pht[4],
+                     "phase_ms": {"moments": pht[1], "chemistry": pht[2], "gradients": pht[3], "energy_collision": pht[4],
                                   "species_collision": pht[5]},
                      "note": "LBM_MIXED with LBM_TRANSPORT_MIXTURE_AVERAGED (Wilke viscosity, Eucken/Mathur "
                              "conductivity, power-law diffusivities per node)"}

@@ -74,10 +74,11 @@ enum { LBM_RXN_ELEMENTARY = 0, LBM_RXN_THIRD_BODY = 1, LBM_RXN_FALLOFF = 2 };
  *                   Stefan-Maxwell solve, the reaction rates and the
  *                   equilibrium constants;
  *   LBM_MIXED_FAST  as LBM_MIXED, but the relaxation rates and the
- *                   Stefan-Maxwell solve run in float and the exponentials
- *                   of the rate expressions take a double range reduction
- *                   with a float 2^f (relative error ~3e-7); its results
- *                   are stored as floats in both mixed modes.  Same
+ *                   Stefan-Maxwell solve run in float, and the exponentials
+ *                   of the reported rates (and of a step's, for mechanisms
+ *                   beyond the fixed-point range: |ln A| >= 512) take a
+ *                   double range reduction with a float 2^f (relative error
+ *                   ~3e-7).  Same
  *                   storage layout and accuracy bar as LBM_MIXED. */
 typedef struct {
     int nx, ny, nz;
