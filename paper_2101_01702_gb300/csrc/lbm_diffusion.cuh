@@ -36,6 +36,7 @@ __device__ __forceinline__ float pow2f(int k)
     return __int_as_float((min(max(k, -126), 127) + 127) << 23);
 }
 
+// 1/x for normal x (the instruction takes subnormal operands for zero).
 __device__ __forceinline__ float rcp_approx(float x)
 {
 #ifdef __CUDA_ARCH__
@@ -43,8 +44,29 @@ __device__ __forceinline__ float rcp_approx(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 #else
-    return 1.0f / x;
+    return 1.0f / (((__float_as_int(x) >> 23) & 0xff) == 0 ? 0.0f * x : x);
 #endif
+}
+
+// 2^k for any k of a double's range, as two factors of a product.
+__device__ __forceinline__ float scale2f(float x, int k)
+{
+    const int k1 = min(max(k, -126), 127);
+    return x * pow2f(k1) * pow2f(k - k1);
+}
+
+// |r| 2^-k in [1, 2) with r's sign as a float of its leading 24 bits and one
+// of the next 23, and k; false for r = 0 or below the normal doubles.
+__device__ __forceinline__ bool mantissa2(double r, float &h, float &l, int &k)
+{
+    const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r), sign = hi & 0x80000000u;
+    const int e = (int)((hi >> 20) & 0x7ffu);
+    const unsigned e2 = sign | (104u << 23);                         // 2^-23
+    h = __uint_as_float(sign | (127u << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+    l = __uint_as_float(e2 | ((lo & 0x1fffffffu) >> 6)) - __uint_as_float(e2);
+    if (e == 0x7ff) h = __int_as_float(0x7fc00000);                  // infinite, NaN
+    k = e - 1023;
+    return e != 0;
 }
 
 // du[M][3], and ita = 1/tau_a [M], of a node, from the rows (stride N) of
@@ -165,14 +187,16 @@ __device__ __forceinline__ void diffusion_refined(const MechConst &mc, const dou
         split2(ud[d * N], uh, ul);
 #pragma unroll
         for (int s = 0; s < M; ++s) {
+            // the quotient of the mantissas: rho_a may be far below the floats
+            // while j_a is not (a trace's rest population is a double)
             float rh, rl;
-            split2(ra[(size_t)s * N], rh, rl);
-            const float j = J[(size_t)(3 * s + d) * N];
+            int k;
+            const bool here = mantissa2(ra[(size_t)s * N], rh, rl, k);
+            const float j = scale2f(J[(size_t)(3 * s + d) * N], -k);
             const float ri = rcp_approx(rh), q = j * ri;
             const float q1 = fma(-q, rl, fma(-q, rh, j)) * ri;
             float e;
             const float s1 = two_sum(q, -uh, e);
-            const bool here = rh != 0.0f;
             Vh[s] = here ? s1 : 0.0f;
             Vl[s] = here ? e + (q1 - ul) : 0.0f;
             x[s] = Vh[s] + Vl[s];
