@@ -11,15 +11,21 @@
 //   d_k = e_k + sum_{j>k} A_kj Y_j            (e = 1/h at the start),
 // sums of positive terms only (Grassmann, Taksar and Heyman's elimination),
 // so the float factors carry a few units of 2^-24 in every entry, however
-// small the mass fractions.  The float solution x0, rounded to integers below
-// 2^29, is an exact operand of the residual
+// small the mass fractions.  The float solution x0 is an exact operand of the
+// residual
 //   r_a = V_a - x_a - (h/W_a) (x_a S_a - sum_b K_ab n_b x_b),
 //   S_a = sum_b K_ab n_b,  K_ab = 1/D_ab,  n_b = Y_b/W_b,
-// whose sums over b run in 58-bit limbs (S_a and the last differences in
-// pairs of floats), 2^-45 of their largest term; the correction, solved with the same
-// factors, is then good to 2^-40 of x, and x0 plus it is rounded to float
-// once -- the float that the double solution rounds to, but for ties
-// (tests/test_diffusion_host.py measures both against a 128-bit solution).
+// whose sums over b run in 58-bit limbs, the products n_b x_b brought to the
+// largest one's exponent, and whose other terms are pairs of floats (2^-46 of
+// each); the correction is solved with the same factors and x0 plus it rounded
+// to float once.  A velocity is the exact one to 2^-40 of the largest
+// n_b |x_b| over the largest n_b and 2^-45 of |u|, rounded to float
+// (tests/test_diffusion_host.py and test_diffusion_traces.py measure it
+// against a 113-bit solution).  Of the velocities of ordinary mixtures
+// 0.03 % are not the float next to the exact one (root mean square error
+// 0.290 units in the last place, 0.289 for exact rounding and for a double
+// LDL^T solve); one that cancels to less than 2^-22 of u or of the others
+// keeps fewer bits than the double solve's.
 //
 // A double LDL^T solve costs 740 FP64 instructions per warp at nine species,
 // 56 thousand cycles of a scheduler; this one about 7 thousand
@@ -79,33 +85,20 @@ __device__ __forceinline__ void diffusion_refined(const MechConst &mc, const dou
                                                   const float *J, size_t N, double hk, double *sh, int bs,
                                                   float (*du)[3], float *ita, bool *bad)
 {
-    // n_b = rho_b / W_b as limbs
-    int en = 0;
+    // n_b = rho_b / W_b
     long long *ln = reinterpret_cast<long long *>(sh), *lS = ln + M * bs;
     float y[M], nh[M], nl[M];
-    unsigned major = 0;                                    // species above 2^-16 of the largest n
-    {
-        double nb[M];
 #pragma unroll
-        for (int b = 0; b < M; ++b) {
-            const double r = ra[(size_t)b * N];
-            nb[b] = r * mc.invW[b];
-            en = max(en, biased_exponent(nb[b]));
-            float lo;
-            split2(r, y[b], lo);
-            y[b] += lo;
-        }
-#pragma unroll
-        for (int b = 0; b < M; ++b) {
-            split2(nb[b], nh[b], nl[b]);
-            const Limbs58 x = to_limbs58(nb[b], en);
-            ln[b * bs] = ((long long)x.h << 32) | (unsigned)x.l;
-            if (biased_exponent(nb[b]) + 16 >= en) major |= 1u << b;
-        }
+    for (int b = 0; b < M; ++b) {
+        const double r = ra[(size_t)b * N], nb = r * mc.invW[b];
+        float lo;
+        split2(r, y[b], lo);
+        y[b] += lo;
+        split2(nb, nh[b], nl[b]);
+        ln[b * bs] = ((long long)__double2hiint(nb) << 32) | (unsigned)__double2loint(nb);
     }
     float hh, hl;
     split2(hk, hh, hl);
-    const int cs = mc.mix_exp + en - 1080 + 58;            // sums of K n are integers times 2^cs
 
     // S_a as pairs of floats, summed with their errors (all terms have one
     // sign, so each S_a keeps its relative accuracy), and 1/tau_a = 2 (h/W_a) S_a
@@ -202,32 +195,29 @@ __device__ __forceinline__ void diffusion_refined(const MechConst &mc, const dou
             x[s] = Vh[s] + Vl[s];
         }
         solve(x);
-        // x0 as integers below 2^29 times 2^-kx, the scale set by the largest
-        // x of a major species; a minor species beyond it by a factor 2^f
-        // takes 2^(f-kx), and starts from zero if its n x0 is beyond the
-        // scale of the sums
-        int em = 0;
+        // w_b = n_b x0_b as integers below 2^58, in units of 2^(ew - 1206), of
+        // which the largest keeps at least 57 bits: from the 53 bits of n_b and
+        // the 24 of x0_b, so that a trace whose momentum balances that of all
+        // others counts in full (subnormal floats x0 count as zero)
+        int ew = 1022 - mc.mix_exp;                                           // sums in units of at least 2^-126
 #pragma unroll
-        for (int s = 0; s < M; ++s)
-            if (major >> s & 1u) em = max(em, (__float_as_int(x[s]) >> 23) & 0xff);
-        const int e0 = min(max(em, 65), 200), kx = 155 - e0;                  // |x0| < 2^(e0 - 126)
-        const int c = cs + 30 - kx;                                           // the sums are integers times 2^c
-        const float g1 = pow2f(41 + c), g2 = pow2f(18 + c), g3 = c < -126 ? 0.0f : pow2f(c);
+        for (int s = 0; s < M; ++s) {
+            const int ex = (__float_as_int(x[s]) >> 23) & 0xff, en = (int)(ln[s * bs] >> 52) & 0x7ff;
+            if (ex == 0) x[s] = 0.0f;
+            if (ex != 0 && en != 0) ew = max(ew, ex + en);
+        }
+        const int c = mc.mix_exp + ew - 1148;                                 // the sums are integers times 2^c
+        const float g1 = pow2f(41 + c), g2 = pow2f(18 + c), g3 = pow2f(c);
         Limbs58 w[M];
 #pragma unroll
         for (int s = 0; s < M; ++s) {
-            const int e = (__float_as_int(x[s]) >> 23) & 0xff, f = min(max(e - e0, 0), 41);
-            int xi = __float2int_rn(x[s] * pow2f(kx - f));
-            const long long v = ln[s * bs];
-            long long ph = (long long)opaque((int)(v >> 32)) * xi, pl = (long long)opaque((int)v) * xi;
-            if (f > 0 && (f > 40 || ((ph < 0 ? -ph : ph) >> (58 - f)) != 0)) {
-                xi = 0;
-                ph = pl = 0;
-            }
-            const long long p = f == 0 ? (ph >> 1) + (pl >> 30)
-                                       : (ph << (f - 1)) + (f <= 30 ? pl >> (30 - f) : pl << (f - 30));
-            w[s] = limbs_of(p);
-            x[s] = (float)xi * pow2f(f - kx);
+            const int xi = __float_as_int(x[s]), hi = opaque((int)(ln[s * bs] >> 32)), lo = opaque((int)ln[s * bs]);
+            const int ex = (xi >> 23) & 0xff, en = (hi >> 20) & 0x7ff;
+            const unsigned mx = ((unsigned)xi & 0x7fffffu) | 0x800000u;
+            const unsigned mh = (((unsigned)hi & 0xfffffu) | 0x100000u) << 8 | (unsigned)lo >> 24, ml = (unsigned)lo & 0xffffffu;
+            const unsigned long long v = ((unsigned long long)mh * mx << 5) + ((unsigned long long)ml * mx >> 19);
+            const long long p = ex != 0 && en != 0 ? (long long)(v >> min(ew - ex - en, 63)) : 0ll;
+            w[s] = limbs_of((hi ^ xi) < 0 ? -p : p);
         }
         float r[M];
 #pragma unroll

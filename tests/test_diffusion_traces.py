@@ -1,7 +1,13 @@
 """The float-refined Stefan-Maxwell solve of the mixed unit, compiled for the
-host, for species far below the others (densities from the smallest subnormal
-double to the normal floats and about the smallest float): every velocity is
-finite."""
+host, for species far below the others: densities from the smallest subnormal
+double to the normal floats (mode 0) and about the smallest float (3), and
+one trace that alone moves, so that its momentum balances the others' (1).
+Every velocity is finite and the exact one to 2^-24 |x| (rounded to float
+once) plus 2^-40 of the largest n_b |x_b| over the largest n_b (the residual
+sums products n_b x_b in integers, 2^-53 of the largest, and takes its other
+terms as pairs of floats, 2^-46 of each; the float correction adds 2^-22 of
+itself) plus 2^-45 |u| (the pairs of floats that hold j/rho and u) plus
+2^-100 (the floats' range)."""
 import os
 import shutil
 import subprocess
@@ -25,9 +31,10 @@ def program(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("mode", [0, 3])
+@pytest.mark.parametrize("mode", [0, 1, 3])
 def test_refined_solve_with_traces(program, mode):
     r = subprocess.run([str(program), str(mode), "4000", str(7 + mode)], capture_output=True, text=True)
     assert r.returncode == 0, r
     nonfinite, worst = (float(v) for v in r.stdout.split())
     assert nonfinite == 0
+    assert worst <= 1.0
