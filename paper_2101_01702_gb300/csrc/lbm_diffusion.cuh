@@ -54,7 +54,17 @@ __device__ __forceinline__ float rcp_approx(float x)
 #endif
 }
 
-// 2^k for any k of a double's range, as two factors of a product.
+// d 2^k; 0 below the normal doubles, d itself if infinite or NaN.  No result
+// may be above the largest double.
+__device__ __forceinline__ double scale2(double d, int k)
+{
+    const long long v = ((long long)__double2hiint(d) << 32) | (unsigned)__double2loint(d);
+    const int e = (int)(v >> 52) & 0x7ff;
+    if (e == 0x7ff) return d;
+    return __longlong_as_double(e == 0 || e + k <= 0 ? 0ll : v + ((long long)k << 52));
+}
+
+// x 2^k for any k of a double's range.
 __device__ __forceinline__ float scale2f(float x, int k)
 {
     const int k1 = min(max(k, -126), 127);
@@ -88,17 +98,24 @@ __device__ __forceinline__ void diffusion_refined(const MechConst &mc, const dou
     // n_b = rho_b / W_b
     long long *ln = reinterpret_cast<long long *>(sh), *lS = ln + M * bs;
     float y[M], nh[M], nl[M];
+    int top = 0;                                           // exponent of the largest
 #pragma unroll
     for (int b = 0; b < M; ++b) {
-        const double r = ra[(size_t)b * N], nb = r * mc.invW[b];
-        float lo;
-        split2(r, y[b], lo);
-        y[b] += lo;
-        split2(nb, nh[b], nl[b]);
+        const double nb = ra[(size_t)b * N] * mc.invW[b];
+        top = max(top, biased_exponent(nb));
         ln[b * bs] = ((long long)__double2hiint(nb) << 32) | (unsigned)__double2loint(nb);
     }
+    // the floats take all densities 2^k times larger, of order one
+    const int k = 1023 - top;
+#pragma unroll
+    for (int b = 0; b < M; ++b) {
+        float lo;
+        split2(scale2(ra[(size_t)b * N], k), y[b], lo);
+        y[b] += lo;
+        split2(scale2(__longlong_as_double(ln[b * bs]), k), nh[b], nl[b]);
+    }
     float hh, hl;
-    split2(hk, hh, hl);
+    split2(scale2(hk, -k), hh, hl);
 
     // S_a as pairs of floats, summed with their errors (all terms have one
     // sign, so each S_a keeps its relative accuracy), and 1/tau_a = 2 (h/W_a) S_a
@@ -183,9 +200,9 @@ __device__ __forceinline__ void diffusion_refined(const MechConst &mc, const dou
             // the quotient of the mantissas: rho_a may be far below the floats
             // while j_a is not (a trace's rest population is a double)
             float rh, rl;
-            int k;
-            const bool here = mantissa2(ra[(size_t)s * N], rh, rl, k);
-            const float j = scale2f(J[(size_t)(3 * s + d) * N], -k);
+            int er;
+            const bool here = mantissa2(ra[(size_t)s * N], rh, rl, er);
+            const float j = scale2f(J[(size_t)(3 * s + d) * N], -er);
             const float ri = rcp_approx(rh), q = j * ri;
             const float q1 = fma(-q, rl, fma(-q, rh, j)) * ri;
             float e;
@@ -199,14 +216,14 @@ __device__ __forceinline__ void diffusion_refined(const MechConst &mc, const dou
         // which the largest keeps at least 57 bits: from the 53 bits of n_b and
         // the 24 of x0_b, so that a trace whose momentum balances that of all
         // others counts in full (subnormal floats x0 count as zero)
-        int ew = 1022 - mc.mix_exp;                                           // sums in units of at least 2^-126
+        int ew = 1022 - mc.mix_exp - k;                                        // sums in units of at least 2^-126
 #pragma unroll
         for (int s = 0; s < M; ++s) {
             const int ex = (__float_as_int(x[s]) >> 23) & 0xff, en = (int)(ln[s * bs] >> 52) & 0x7ff;
             if (ex == 0) x[s] = 0.0f;
             if (ex != 0 && en != 0) ew = max(ew, ex + en);
         }
-        const int c = mc.mix_exp + ew - 1148;                                 // the sums are integers times 2^c
+        const int c = mc.mix_exp + ew + k - 1148;                                // the sums are integers times 2^c
         const float g1 = pow2f(41 + c), g2 = pow2f(18 + c), g3 = pow2f(c);
         Limbs58 w[M];
 #pragma unroll

@@ -1,7 +1,8 @@
 """The float-refined Stefan-Maxwell solve of the mixed unit, compiled for the
 host, for species far below the others: densities from the smallest subnormal
 double to the normal floats (mode 0) and about the smallest float (3), and
-one trace that alone moves, so that its momentum balances the others' (1).
+one trace that alone moves, so that its momentum balances the others' (1);
+and for another unit of density, 2^-70 to 2^70 times the first (2).
 Every velocity is finite and the exact one to 2^-24 |x| (rounded to float
 once) plus 2^-40 of the largest n_b |x_b| over the largest n_b (the residual
 sums products n_b x_b in integers, 2^-53 of the largest, and takes its other
@@ -31,7 +32,7 @@ def program(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("mode", [0, 1, 3])
+@pytest.mark.parametrize("mode", [0, 1, 2, 3])
 def test_refined_solve_with_traces(program, mode):
     r = subprocess.run([str(program), str(mode), "4000", str(7 + mode)], capture_output=True, text=True)
     assert r.returncode == 0, r
