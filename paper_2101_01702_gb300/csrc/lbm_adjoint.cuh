@@ -400,7 +400,7 @@ __device__ void adj_collide_node(const MechConst &mc, const StepArgs &a, const A
             for (int j = 0; j < k; ++j) sacc = fma(-Ln[i][j], Dk[j], sacc);
             Ln[i][k] = sacc;
         }
-        Dinv[k] = nonzero_bits(Ln[k][k]) ? 1.0 / Ln[k][k] : 0.0;
+        Dinv[k] = invertible_bits(Ln[k][k]) ? 1.0 / Ln[k][k] : 0.0;
 #pragma unroll
         for (int i = k + 1; i < M; ++i) Ln[i][k] *= Dinv[k];
     }

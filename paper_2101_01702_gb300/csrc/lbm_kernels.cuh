@@ -165,14 +165,12 @@ __device__ __forceinline__ int wrapi(int v, int n) { return v < 0 ? v + n : (v >
 __device__ __forceinline__ void flag(unsigned *status, unsigned bit) { atomicOr(status, bit); }
 
 // Tests on the bit pattern (integer pipe; the FP64 pipe is the step's
-// bottleneck): not Inf or NaN, and not +-0.
+// bottleneck): not Inf or NaN, and of a magnitude whose reciprocal is finite
+// (above 2^-1024 and 2^-128; true for NaN).
 __device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 __device__ __forceinline__ bool finite_bits(float x) { return (__float_as_int(x) & 0x7f800000) != 0x7f800000; }
-__device__ __forceinline__ bool nonzero_bits(double x)
-{
-    return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) != 0;
-}
-__device__ __forceinline__ bool nonzero_bits(float x) { return (__float_as_int(x) & 0x7fffffff) != 0; }
+__device__ __forceinline__ bool invertible_bits(double x) { return (__double2hiint(x) & 0x7fffffff) > 0x00040000; }
+__device__ __forceinline__ bool invertible_bits(float x) { return (__float_as_int(x) & 0x7fffffff) > 0x00200000; }
 
 // Conversions between float and double on the integer pipe.  A hardware
 // conversion between the two issues on the FP64 pipe, which bounds the
@@ -1774,9 +1772,11 @@ __device__ __forceinline__ void diff_node(const StepArgs &a, const Node &nd, dou
             // to a rounding-level negative density, zero only for an absent
             // species (Y_k = 0), whose row and column vanish and whose
             // diffusion velocity is multiplied by Y_k = 0 wherever it is used.
+            // A species so far below the others that 1/D_k would be infinite
+            // counts as absent.
             D[k] = Ln[k][k];
             if (!finite_bits(D[k])) flag(a.status, LBMK_BIT_PIVOT);
-            Dinv[k] = nonzero_bits(D[k]) ? (SReal)1 / D[k] : (SReal)0;
+            Dinv[k] = invertible_bits(D[k]) ? (SReal)1 / D[k] : (SReal)0;
 #pragma unroll
             for (int i = k + 1; i < M; ++i) Ln[i][k] *= Dinv[k];
         }

@@ -48,7 +48,7 @@ def reference(lbm, problem):
 
 
 @pytest.mark.parametrize("launch", ["kernels", "persistent"])
-@pytest.mark.parametrize("mode", ["mixed"])
+@pytest.mark.parametrize("mode", ["mixed", "mixed_fast"])
 def test_species_from_zero(lbm, problem, reference, mode, launch):
     s = lbm.Solver.from_problem(problem, precision=lbm.LBM_MIXED if mode == "mixed" else lbm.LBM_MIXED_FAST)
     if launch == "kernels":
