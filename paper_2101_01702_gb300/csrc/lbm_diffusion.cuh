@@ -36,12 +36,6 @@
 
 namespace {
 
-// 2^k, clamped to the normal floats.
-__device__ __forceinline__ float pow2f(int k)
-{
-    return __int_as_float((min(max(k, -126), 127) + 127) << 23);
-}
-
 // 1/x for normal x (the instruction takes subnormal operands for zero).
 __device__ __forceinline__ float rcp_approx(float x)
 {
@@ -52,16 +46,6 @@ __device__ __forceinline__ float rcp_approx(float x)
 #else
     return 1.0f / (((__float_as_int(x) >> 23) & 0xff) == 0 ? 0.0f * x : x);
 #endif
-}
-
-// d 2^k; 0 below the normal doubles, d itself if infinite or NaN.  No result
-// may be above the largest double.
-__device__ __forceinline__ double scale2(double d, int k)
-{
-    const long long v = ((long long)__double2hiint(d) << 32) | (unsigned)__double2loint(d);
-    const int e = (int)(v >> 52) & 0x7ff;
-    if (e == 0x7ff) return d;
-    return __longlong_as_double(e == 0 || e + k <= 0 ? 0ll : v + ((long long)k << 52));
 }
 
 // x 2^k for any k of a double's range.

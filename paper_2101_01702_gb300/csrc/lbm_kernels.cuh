@@ -1165,50 +1165,6 @@ __device__ __forceinline__ long long shift_by(long long v, int sh)
     return sh >= 0 ? (long long)((unsigned long long)v << (sh & 63)) : v >> (sh < -63 ? 63 : -sh);
 }
 
-// Sums of the molar production rates, one 8-byte column per species: in
-// double, or (PAIR) in pairs of floats, for callers that store the rates as
-// floats: a sum and the sum of its rounding errors (two_sum), 48 bits.
-template <bool PAIR>
-struct RateSums {
-    double *col;
-    int stride;
-    __device__ __forceinline__ void clear(int s) { col[s * stride] = 0.0; }
-    struct Term {
-        double q;
-        float h, l;
-    };
-    __device__ __forceinline__ Term term(double q) const
-    {
-        Term t{q, 0.0f, 0.0f};
-        if (PAIR) split2(q, t.h, t.l);
-        return t;
-    }
-    template <int SIGN>
-    __device__ __forceinline__ void add(int s, const Term &t)
-    {
-        if (PAIR) {
-            float2 *p = reinterpret_cast<float2 *>(col + s * stride);
-            float2 v = *p;
-            float e;
-            v.x = two_sum(v.x, SIGN * t.h, e);
-            v.y += e + SIGN * t.l;
-            *p = v;
-        } else {
-            col[s * stride] += SIGN * t.q;
-        }
-    }
-    // w_s times the molar mass
-    __device__ __forceinline__ double mass(int s, double W) const { return W * col[s * stride]; }
-    __device__ __forceinline__ float mass_float(int s, double W) const
-    {
-        const float2 v = *reinterpret_cast<const float2 *>(col + s * stride);
-        float wh, wl;
-        split2(W, wh, wl);
-        const float p = wh * v.x;
-        return p + (fma(wh, v.x, -p) + fma(wh, v.y, wl * v.x));
-    }
-};
-
 // Molar production rates as molar_production below forms them, with every
 // exponent an integer sum in units of 2^-53: the Gibbs functions
 //   g_a/(R_U T) = sum_j gco_aj phi_j,  phi = 1 - ln T, T .. T^4, 1/T, 1,
@@ -1379,7 +1335,7 @@ __device__ __forceinline__ void production_rates(const MechConst &mc, double T, 
 {
 #if !LBMK_FAST
     if (mc.chem_fixed) {
-        molar_production_fixed<M, false>(mc, T, conc, sh_act, sh_g, RateSums<false>{sh_w + t, stride}, t, stride);
+        molar_production_fixed<M, false>(mc, T, conc, sh_act, sh_g, RateSums<false>{sh_w + t, stride, 0}, t, stride);
         return;
     }
 #endif
@@ -1876,7 +1832,7 @@ __device__ __forceinline__ void chem_node(const StepArgs &a, int n, double *sh, 
     Real *wd = R + (size_t)rr.wd * N + n;
 #if LBMK_MIXED
     if (mc.chem_fixed) {
-        const RateSums<true> w{sh + 2 * M * bs + t, bs};
+        const RateSums<true> w{sh + 2 * M * bs + t, bs, rate_scale(rho)};
         molar_production_fixed<M, true>(mc, T, conc, sh_act, sh_g, w, t, bs);
 #pragma unroll
         for (int s = 0; s < M; ++s) wd[(size_t)s * N] = w.mass_float(s, mc.W[s]);
