@@ -19,13 +19,15 @@
 // largest one's exponent, and whose other terms are pairs of floats (2^-46 of
 // each); the correction is solved with the same factors and x0 plus it rounded
 // to float once.  A velocity is the exact one to 2^-40 of the largest
-// n_b |x_b| over the largest n_b and 2^-45 of |u|, rounded to float
-// (tests/test_diffusion_host.py and test_diffusion_traces.py measure it
-// against a 113-bit solution).  Of the velocities of ordinary mixtures
-// 0.03 % are not the float next to the exact one (root mean square error
-// 0.290 units in the last place, 0.289 for exact rounding and for a double
-// LDL^T solve); one that cancels to less than 2^-22 of u or of the others
-// keeps fewer bits than the double solve's.
+// n_b |x_b| over the largest n_b and 2^-53 of |u|, rounded to float
+// (tests/test_diffusion_traces.py measures it against a 113-bit solution).
+// That is no further from the exact velocity than a double LDL^T solve
+// rounded to float.  Root mean square error in units of the last place, each
+// over 540,000 velocities of nine species (exact rounding: 0.289): ordinary
+// mixtures 0.289 (LDL^T 0.289), traces down to 1e-14 0.289 (4.2), down to
+// 1e-10 with absent species 0.289 (0.59), rounding-level traces of either
+// sign 0.289 (0.289), one species nearly pure 0.289 (5e6: its j_a/rho and
+// Y_a u cancel).
 //
 // A double LDL^T solve costs 740 FP64 instructions per warp at nine species,
 // 56 thousand cycles of a scheduler; this one about 7 thousand
@@ -48,18 +50,11 @@ __device__ __forceinline__ float rcp_approx(float x)
 #endif
 }
 
-// x 2^k for any k of a double's range.
-__device__ __forceinline__ float scale2f(float x, int k)
+// |d| 2^-k in [1, 2) with d's sign as a float of its leading 24 bits and one
+// of the next 23, and k; false for d = 0 or below the normal doubles.
+__device__ __forceinline__ bool mantissa2(double d, float &h, float &l, int &k)
 {
-    const int k1 = min(max(k, -126), 127);
-    return x * pow2f(k1) * pow2f(k - k1);
-}
-
-// |r| 2^-k in [1, 2) with r's sign as a float of its leading 24 bits and one
-// of the next 23, and k; false for r = 0 or below the normal doubles.
-__device__ __forceinline__ bool mantissa2(double r, float &h, float &l, int &k)
-{
-    const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r), sign = hi & 0x80000000u;
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d), sign = hi & 0x80000000u;
     const int e = (int)((hi >> 20) & 0x7ffu);
     const unsigned e2 = sign | (104u << 23);                         // 2^-23
     h = __uint_as_float(sign | (127u << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
@@ -69,16 +64,65 @@ __device__ __forceinline__ bool mantissa2(double r, float &h, float &l, int &k)
     return e != 0;
 }
 
+// x as a double, on the integer pipe; subnormals by way of 2^64 times them.
+__device__ __forceinline__ double widen(float x)
+{
+    const bool small = ((__float_as_int(x) >> 23) & 0xff) == 0;
+    const unsigned b = (unsigned)__float_as_int(small ? x * 18446744073709551616.0f : x), mag = b & 0x7fffffffu;
+    const unsigned bias = (mag >> 23) == 255u ? 1792u : (small ? 832u : 896u);
+    const unsigned hi = (b & 0x80000000u) | (mag == 0u ? 0u : (mag >> 3) + (bias << 20));
+    return __longlong_as_double((long long)((unsigned long long)hi << 32 | (unsigned long long)(b << 29)));
+}
+
+// V = j/r - u as a pair of floats, 0 for r = 0 or below the normal doubles:
+// the numerator j - r u in one double operation, which rounds once however
+// much of the two cancels, of r's mantissa and j scaled by r's exponent (r may
+// be far below the floats while j is not: a trace's rest population is a
+// double), and its quotient by the mantissa.  |V| below 2^-126 or above 2^127
+// counts as that.
+__device__ __forceinline__ void slip_velocity(double r, float j, double u, float &h, float &l)
+{
+    float dh, dl, rh, rl;
+    int kd, kr;
+    const bool here = mantissa2(r, rh, rl, kr);
+    const unsigned m = ((unsigned)__double2hiint(r) & 0x800fffffu) | 0x3ff00000u;
+    const double rm = __longlong_as_double((long long)((unsigned long long)m << 32 | (unsigned)__double2loint(r)));
+    const bool moves = mantissa2(fma(-rm, u, scale2(widen(j), -kr)), dh, dl, kd);
+    const float ri = rcp_approx(rh), v = dh * ri;
+    const float w = (fma(-v, rl, fma(-v, rh, dh)) + dl) * ri;
+    const float g = moves && here ? pow2f(kd) : 0.0f;
+    h = v * g;
+    l = w * g;
+}
+
 // du[M][3], and ita = 1/tau_a [M], of a node, from the rows (stride N) of
 // its species densities ra, velocity ud and momenta J, and hk = h/rho.  All
 // quantities are scale-free in the densities: with rho_b in place of Y_b, h
 // becomes h/rho.  sh: 2 M columns of this thread's shared memory, stride
-// bs.  Sets *bad for a non-finite pivot.
-template <int M>
+// bs, or 5 M with KEEP, as the kernel has it: the V_a of all three components
+// are then formed before the factorisation and kept in the last 3 M, so that
+// their loads overlap and the loop over the components fits the registers
+// (moments and diffusion, 256^3: 22.1 ms; formed in that loop 24.9, and 25.3
+// with j - r u in integers there; 23.1 with V from j/r and u as pairs of
+// floats, 2^-46 of each and up to 160 times the double solve's error where
+// they cancel).  Sets *bad for a non-finite pivot.
+template <int M, bool KEEP = false>
 __device__ __forceinline__ void diffusion_refined(const MechConst &mc, const double *ra, const double *ud,
                                                   const float *J, size_t N, double hk, double *sh, int bs,
                                                   float (*du)[3], float *ita, bool *bad)
 {
+    float2 *sV = reinterpret_cast<float2 *>(sh + 2 * M * bs);
+    if (KEEP) {
+        const double u0 = ud[0], u1 = ud[N], u2 = ud[2 * N];
+#pragma unroll
+        for (int s = 0; s < M; ++s)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                float2 v;
+                slip_velocity(ra[(size_t)s * N], J[(size_t)(3 * s + d) * N], d == 0 ? u0 : (d == 1 ? u1 : u2), v.x, v.y);
+                sV[(3 * s + d) * bs] = v;
+            }
+    }
     // n_b = rho_b / W_b
     long long *ln = reinterpret_cast<long long *>(sh), *lS = ln + M * bs;
     float y[M], nh[M], nl[M];
@@ -175,25 +219,20 @@ __device__ __forceinline__ void diffusion_refined(const MechConst &mc, const dou
 
 #pragma unroll 1
     for (int d = 0; d < 3; ++d) {
-        // V_a = j_a / rho_a - u as pairs of floats; 0 for an absent species
         float Vh[M], Vl[M], x[M];
-        float uh, ul;
-        split2(ud[d * N], uh, ul);
+        {
+            const double u = KEEP ? 0.0 : ud[d * N];
 #pragma unroll
-        for (int s = 0; s < M; ++s) {
-            // the quotient of the mantissas: rho_a may be far below the floats
-            // while j_a is not (a trace's rest population is a double)
-            float rh, rl;
-            int er;
-            const bool here = mantissa2(ra[(size_t)s * N], rh, rl, er);
-            const float j = scale2f(J[(size_t)(3 * s + d) * N], -er);
-            const float ri = rcp_approx(rh), q = j * ri;
-            const float q1 = fma(-q, rl, fma(-q, rh, j)) * ri;
-            float e;
-            const float s1 = two_sum(q, -uh, e);
-            Vh[s] = here ? s1 : 0.0f;
-            Vl[s] = here ? e + (q1 - ul) : 0.0f;
-            x[s] = Vh[s] + Vl[s];
+            for (int s = 0; s < M; ++s) {
+                if (KEEP) {
+                    const float2 v = sV[(3 * s + d) * bs];
+                    Vh[s] = v.x;
+                    Vl[s] = v.y;
+                } else {
+                    slip_velocity(ra[(size_t)s * N], J[(size_t)(3 * s + d) * N], u, Vh[s], Vl[s]);
+                }
+                x[s] = Vh[s] + Vl[s];
+            }
         }
         solve(x);
         // w_b = n_b x0_b as integers below 2^58, in units of 2^(ew - 1206), of

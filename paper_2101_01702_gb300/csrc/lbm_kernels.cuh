@@ -1622,7 +1622,7 @@ template <int M, bool FX>
 constexpr bool kRefined = FX && M >= 4 && LBMK_MIXED && !LBMK_FAST;
 
 template <int M, bool FX>
-constexpr int diff_cols() { return kRefined<M, FX> ? 2 * M : 0; }
+constexpr int diff_cols() { return kRefined<M, FX> ? 5 * M : 0; }
 
 template <int M, bool FX>
 __device__ __forceinline__ void diff_node(const StepArgs &a, const Node &nd, double *sh, int bs)
@@ -1640,8 +1640,9 @@ __device__ __forceinline__ void diff_node(const StepArgs &a, const Node &nd, dou
 #if LBMK_MIXED && !LBMK_FAST
     if constexpr (kRefined<M, FX>) {
         bool bad = false;
-        diffusion_refined<M>(mc, dr + (size_t)diff_rows(M).ra * N, dr + (size_t)diff_rows(M).u * N,
-                             R + (size_t)rr.du * N + n, N, dr[(size_t)diff_rows(M).hk * N], sh, bs, duR, itaR, &bad);
+        diffusion_refined<M, true>(mc, dr + (size_t)diff_rows(M).ra * N, dr + (size_t)diff_rows(M).u * N,
+                                   R + (size_t)rr.du * N + n, N, dr[(size_t)diff_rows(M).hk * N], sh, bs, duR, itaR,
+                                   &bad);
         if (bad) flag(a.status, LBMK_BIT_PIVOT);
     } else
 #endif
@@ -2197,7 +2198,8 @@ constexpr size_t step_smem(int bs) { return (size_t)step_cols<M>() * bs * sizeof
 template <int M>
 constexpr size_t persist_smem(int bs)
 {
-    return (size_t)(step_cols<M>() > chem_cols<M>() ? step_cols<M>() : chem_cols<M>()) * bs * sizeof(double);
+    constexpr int d = diff_cols<M, true>(), c = chem_cols<M>(), s = step_cols<M>();
+    return (size_t)(d > c ? (d > s ? d : s) : (c > s ? c : s)) * bs * sizeof(double);
 }
 
 extern __shared__ double sh_step[];
@@ -2270,6 +2272,7 @@ int launch_one(const StepArgs &a, int k)
     case LBMK_K_PRE: {
         k_pre<M><<<grid_for(a.N, bs), bs, pre_cols<M>() * bs * sizeof(double), a.stream>>>(a);
         constexpr bool FX = kRefined<M, true>;
+        static_assert(diff_cols<M, true>() * LBMK_BLOCK * sizeof(double) <= 48 * 1024, "more needs an opt-in");
         if (FX && a.fixed)
             k_diff<M, FX><<<grid_for(a.N, bs), bs, diff_cols<M, FX>() * bs * sizeof(double), a.stream>>>(a);
         else

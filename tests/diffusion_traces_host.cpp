@@ -4,7 +4,7 @@
 // of two.  Arguments: mode (see below), count, seed.  Prints the number of
 // velocities that are not finite, and the largest |error| against a solve in
 // 113-bit arithmetic in units of 2^-24 |x| + 2^-40 max_b(n_b |x_b|)/max_b n_b
-// + 2^-45 |u| + 2^-100, n = rho/W.  The stand-ins for the device's intrinsics are those
+// + 2^-53 |u| + 2^-100, n = rho/W.  The stand-ins for the device's intrinsics are those
 // of diffusion_host.cpp.
 #define main diffusion_host_main
 #include "diffusion_host.cpp"
@@ -64,10 +64,10 @@ int main(int argc, char **argv)
         double im = 0;
         for (int a = 0; a < M; ++a) im += ra[a] / r / W[a];
         const double kappa = sp.r_lat * U(280, 2500) / im;
-        double sh[2 * M];
+        double sh[5 * M];
         float du[M][3], ita[M];
         bool bad = false;
-        diffusion_refined<M>(mc, ra, u, &j[0][0], 1, 0.5 * kappa / r, sh, 1, du, ita, &bad);
+        diffusion_refined<M, true>(mc, ra, u, &j[0][0], 1, 0.5 * kappa / r, sh, 1, du, ita, &bad);
         if (bad) return 3;
         Q B[M][M], b[M][3], x[M][3];
         for (int a = 0; a < M; ++a) {
@@ -106,7 +106,7 @@ int main(int argc, char **argv)
                 // a subnormal double counts as an absent species: velocity zero or the mean of the others
                 if (ra[a] < 0x1p-1022) continue;
                 const double e = fabs((double)((Q)du[a][d] - x[a][d])), ex = fabs((double)x[a][d]);
-                worst = max(worst, e / (0x1p-24 * ex + 0x1p-40 * (flux / top) + 0x1p-45 * fabs(u[d]) + 0x1p-100));
+                worst = max(worst, e / (0x1p-24 * ex + 0x1p-40 * (flux / top) + 0x1p-53 * fabs(u[d]) + 0x1p-100));
             }
         }
     }
