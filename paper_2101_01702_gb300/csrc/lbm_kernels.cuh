@@ -1148,13 +1148,14 @@ __device__ __forceinline__ double exp_rate(double x)
 #endif
 }
 
-// exp(x) for x in units of 2^-53 (modulo 2^64) and a float within 1e-4 of it;
-// beyond +-707 from the float alone.
+// exp(x) for x in units of 2^-53 (modulo 2^64) and a float within 1e-4 of it.
+// Beyond +-707 exp() itself, of x as far as the unit holds it (e^x is 0 or
+// infinite beyond).
 __device__ __forceinline__ double exp_fixed(long long x, float xf)
 {
     constexpr double kInv = 0x1.71547652b82fep+8, kL1 = 0x1.62e42fefc0000p-9, kL2 = -0x1.c610ca86c3899p-45;
     constexpr long long L1 = (long long)(kL1 * 0x1p+70), L2 = (long long)(kL2 * 0x1p+88);
-    if (!(fabsf(xf) < 707.0f)) return exp((double)xf);
+    if (!(fabsf(xf) < 707.0f)) return exp(fabsf(xf) < 1000.0f ? (double)x * 0x1p-53 : (double)xf);
     const int n = __float_as_int(fmaf(xf, (float)kInv, 12582912.0f)) - 0x4b400000;
     return exp_reduced((unsigned long long)x << 17, n, L1, L2);
 }
