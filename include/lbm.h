@@ -255,17 +255,19 @@ int lbm_autotune_persistent(lbm_ctx *ctx, int steps, int *tile_mult_out);
  * candidate block size -- 64 or 128 threads for the moment and species-
  * collision kernels, whose register budgets are set for 128, and 64, 128
  * or 256 for the production-rate, gradient and energy-collision kernels --
- * over `trials` launches (1..1000) after two untimed ones, and keeps the
- * fastest for every later step of this context.  The state is left as it
+ * and with the choice by the lattice's size that an untuned context has
+ * (down to 32 threads on small lattices), over `trials` launches (1..1000)
+ * after two untimed ones, and keeps the fastest for every later step of
+ * this context.  The state is left as it
  * was (the kernels write only the per-node record and the other buffer;
  * the temperature row, the next Newton start, is restored), so results
  * are bit for bit those of the untuned context.  Allocates and frees one
  * temporary row of N doubles.  block_out (NULL or 6 ints) receives the
  * chosen blocks in launch order: ghost nodes, moments, production rates,
  * gradients, energy collision, species/mixture collision (the moment entry
- * covers the diffusion-velocity kernel as well).  A context that is not
- * tuned takes blocks by the lattice's size.  Waits for the stream; returns
- * like lbm_sync. */
+ * covers the diffusion-velocity kernel as well); for a kernel whose choice
+ * by size is kept, the fastest of the sizes that lbm_set_blocks takes.
+ * Waits for the stream; returns like lbm_sync. */
 int lbm_autotune(lbm_ctx *ctx, int trials, int *block_out);
 
 /* Sets the block sizes of the six kernels directly (for instance a choice

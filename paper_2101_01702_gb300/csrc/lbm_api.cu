@@ -592,7 +592,7 @@ int lbm_autotune(lbm_ctx *c, int trials, int *block_out)
     if (st != LBM_OK) return st;
     // Candidate blocks per kernel: k_pre and k_step carry register caps for
     // 128-thread blocks, so at most 128; the others up to LBMK_MAXBLOCK.
-    static const int cand[3] = {64, 128, 256};
+    int report[LBMK_NKERNELS] = {0};
     const int maxbs[LBMK_NKERNELS] = {LBMK_BLOCK, LBMK_BLOCK, LBMK_MAXBLOCK, LBMK_MAXBLOCK, LBMK_MAXBLOCK,
                                       LBMK_BLOCK};
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -619,27 +619,26 @@ int lbm_autotune(lbm_ctx *c, int trials, int *block_out)
     for (int k = 0; k < LBMK_NKERNELS && st == LBM_OK; ++k) {
         StepArgs a = args_of(c);
         if (op.launch_one(a, k)) { st = LBM_ERR_CUDA; break; }     // the kernel's inputs, at the current choice
-        if (k == LBMK_K_GHOST) continue;
-        float best = 0.f;
-        for (int j = 0; j < 3 && st == LBM_OK; ++j) {
-            if (cand[j] > maxbs[k]) continue;
-            a.bs[k] = cand[j];
+        if (k == LBMK_K_GHOST) {
+            report[k] = c->bs[k];
+            continue;
+        }
+        float ms[LBMK_NBLOCKS] = {0.f};
+        for (int j = 0; j < LBMK_NBLOCKS && st == LBM_OK; ++j) {
+            if (lbmk_block_cand[j] > maxbs[k]) continue;
+            a.bs[k] = lbmk_block_cand[j];
             for (int w = 0; w < 2 + trials && st == LBM_OK; ++w) {   // 2 untimed, then trials timed
                 if (w == 2 && cudaEventRecord(e0, c->stream) != cudaSuccess) st = LBM_ERR_CUDA;
                 if (op.launch_one(a, k)) st = LBM_ERR_CUDA;
             }
             if (st != LBM_OK) break;
-            float ms = 0.f;
             if (cudaEventRecord(e1, c->stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
-                cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
+                cudaEventElapsedTime(&ms[j], e0, e1) != cudaSuccess) {
                 st = LBM_ERR_CUDA;
                 break;
             }
-            if (best == 0.f || ms < best) {
-                best = ms;
-                c->bs[k] = cand[j];
-            }
         }
+        if (st == LBM_OK) c->bs[k] = lbmk_choose_block(ms, &report[k]);
         a = args_of(c);
         if (st == LBM_OK && op.launch_one(a, k)) st = LBM_ERR_CUDA;   // leave its outputs from the choice
     }
@@ -655,7 +654,7 @@ int lbm_autotune(lbm_ctx *c, int trials, int *block_out)
         c->graph = nullptr;
     }
     if (block_out)
-        for (int k = 0; k < LBMK_NKERNELS; ++k) block_out[k] = c->bs[k];
+        for (int k = 0; k < LBMK_NKERNELS; ++k) block_out[k] = report[k];
     if (st != LBM_OK) return st;
     return lbm_sync(c);
 }

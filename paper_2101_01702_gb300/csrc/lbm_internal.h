@@ -193,6 +193,25 @@ static_assert(LBMK_SLOTS * sizeof(MechConst) <= 65536, "four slots have to fit c
 // block sizes are indexed alike).
 enum { LBMK_K_GHOST = 0, LBMK_K_PRE, LBMK_K_CHEM, LBMK_K_GRAD, LBMK_K_STEPG, LBMK_K_STEP, LBMK_NKERNELS };
 
+// The autotuner's candidates for threads per block: 0, the choice by the
+// lattice's size that an untuned context has (down to 32 threads, block_of),
+// and the sizes of lbm_set_blocks.
+#define LBMK_NBLOCKS 4
+constexpr int lbmk_block_cand[LBMK_NBLOCKS] = {0, 64, 128, 256};
+
+// The fastest candidate by the times ms (0: not tried), the choice by size
+// where no other is faster by 2 %, more than the timings of a few launches
+// differ; *fixed: the fastest of the others.  Without the choice by size among
+// the candidates, 48^3 mixed took 452 to 458 us a step tuned and 447 untuned.
+inline int lbmk_choose_block(const float *ms, int *fixed)
+{
+    int best = 0;
+    for (int j = 1; j < LBMK_NBLOCKS; ++j)
+        if (ms[j] > 0.f && (best == 0 || ms[j] < ms[best])) best = j;
+    *fixed = lbmk_block_cand[best];
+    return ms[0] > 0.f && (best == 0 || ms[0] <= 1.02f * ms[best]) ? lbmk_block_cand[0] : lbmk_block_cand[best];
+}
+
 struct StepArgs {
     int slot, M, nx, ny, nz, N, bc_x;
     int fixed;               // the tables' mix_fixed: kernels with fixed-point sums over the species
