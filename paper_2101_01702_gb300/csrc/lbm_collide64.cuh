@@ -15,10 +15,11 @@
 // limbs, each block brought to its largest exponent, and K to that of its
 // largest entry.
 //
-// Measured, 128^3 with nine species, rates included: 33.2 ms with every
-// term formed per direction in floating point; 15.4 ms with the D_b in double
-// and only the sums over b in integers (14.1 ms after the exponentials left
-// the FP64 pipe); 1024 nodes with three species: 101 -> 53 us.
+// Measured, 128^3 with nine species: with the production rates in the kernel
+// 33.2 ms with every term formed per direction in floating point, 15.4 with
+// the D_b in double and only the sums over b in integers, 13.1 with both in
+// integers, 11.1 after the exponentials and exponents of the rates left the
+// FP64 pipe; without the rates (a kernel of 1.5 ms of its own) 8.0 ms.
 #pragma once
 
 #include "lbm_fixed.cuh"

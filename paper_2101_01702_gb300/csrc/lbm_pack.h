@@ -135,8 +135,8 @@ static inline int lbm_pack_tables(const lbm_species *sp, const lbm_mechanism *me
                     top = fmax(top, 1.0 / sp->D[M * a + b]);
                     low = fmin(low, 1.0 / sp->D[M * a + b]);
                 }
-        const int e = isfinite(top) ? ilogb(top) : 0;
-        mc.mix_fixed = M <= LBMK_MIXM && isfinite(top) && top <= 32.0 * low && e >= -12 && e <= 20;
+        const int e = isfinite(top) && top > 0.0 ? ilogb(top) : 0;
+        mc.mix_fixed = isfinite(top) && top <= 32.0 * low && top >= 0x1p-12 && e <= 20;
         for (int a = 0; a < M; ++a) {
             if (sp->W[a] < 0x1p-12 || sp->W[a] > 0x1p+12) mc.mix_fixed = 0;
             mc.invW_h[a] = (float)mc.invW[a];
