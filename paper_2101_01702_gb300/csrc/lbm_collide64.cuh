@@ -12,14 +12,15 @@
 // its row, two multiply-adds).  The differences D_b and the sums over the
 // partner species -- (M-1)^2 terms per direction -- run on the integer pipe
 // (lbm_fixed.cuh): the y-z parts of a row and the x factors of a direction as
-// limbs, each block brought to its largest exponent, and K to that of its
-// largest entry.
+// limbs at each species' own exponent, the D_b brought to the largest one's,
+// and K to that of its largest entry.
 //
 // Measured, 128^3 with nine species: with the production rates in the kernel
 // 33.2 ms with every term formed per direction in floating point, 15.4 with
 // the D_b in double and only the sums over b in integers, 13.1 with both in
 // integers, 11.1 after the exponentials and exponents of the rates left the
-// FP64 pipe; without the rates (a kernel of 1.5 ms of its own) 8.0 ms.
+// FP64 pipe; without the rates (a kernel of 1.5 ms of its own) 8.0 ms,
+// 8.2 with each species' own exponents (limb_differences).
 #pragma once
 
 #include "lbm_fixed.cuh"
@@ -79,6 +80,7 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
     const double u[3] = {ld(rr.u), ld(rr.u + 1), ld(rr.u + 2)};
     const double om = ld(rr.om), omf = 1.0 - om, omr = om * rho, RT = ld(rr.rt);
     int ex[3] = {0, 0, 0};                                  // exponents of the x factors, per c
+    Below dx[3] = {0, 0, 0};
     double fx[3];                                           // x factors of the mixture set
     {
         PsiCoef q[2][3];
@@ -113,7 +115,9 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     double *x = sh + (size_t)(12 * s + 9 + c) * bs + t;
-                    const Limbs58 v = to_limbs58(*x, ex[c]);
+                    const int e = max(biased_exponent(x[-3 * bs]), biased_exponent(*x));
+                    dx[c] |= below_field(s, ex[c], e);
+                    const Limbs58 v = to_limbs58(*x, ex[c] - below_of(dx[c], s));
                     *x = __hiloint2double(v.h, v.l);
                 }
         }
@@ -167,11 +171,14 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
                 er = max(er, max(biased_exponent(pe[s]), biased_exponent(ps[s])));
             }
             Limbs58 le[M], ls[M];
+            Below dr = 0;
             if constexpr (FX) {
 #pragma unroll
                 for (int s = 0; s < M; ++s) {
-                    le[s] = to_limbs58(pe[s], er);
-                    const Limbs58 x = to_limbs58(ps[s], er);
+                    dr |= below_field(s, er, max(biased_exponent(pe[s]), biased_exponent(ps[s])));
+                    const int e = er - below_of(dr, s);
+                    le[s] = to_limbs58(pe[s], e);
+                    const Limbs58 x = to_limbs58(ps[s], e);
                     ls[s] = Limbs58{opaque(-x.h), opaque(-x.l)};
                     if (s < M - 1) pe[s] *= kE[s];
                 }
@@ -195,18 +202,18 @@ __device__ __forceinline__ void step_node(const StepArgs &a, const Node &nd, dou
                 if constexpr (FX) {
                     const int exc = cx < 0 ? ex[0] : (cx == 0 ? ex[1] : ex[2]);
                     Limbs58 D[M];
-#pragma unroll
-                    for (int s = 0; s < M; ++s) {
-                        const double xe = sh[(12 * s + 6 + cx + 1) * bs + t], xs = sh[(12 * s + 9 + cx + 1) * bs + t];
-                        E[s] = pe[s] * xe;                     // (2 beta_a rho_a + rho_dot_a) e_a; not used for the last
-                        const Limbs58 l = to_limbs58(xe, exc), m{__double2hiint(xs), __double2loint(xs)};
-                        long long hi = 0, mid = 0;
-                        fma_limbs58(hi, mid, le[s], l);
-                        fma_limbs58(hi, mid, ls[s], m);
-                        const long long d = hi + (mid >> 29);  // below 2^59
-                        D[s] = limbs_of(d);
-                    }
-                    const int e = er + exc - 2044 + mc.mix_exp;
+                    const int least = limb_differences<M>(
+                        le, ls, dr, cx < 0 ? dx[0] : (cx == 0 ? dx[1] : dx[2]), exc,
+                        [&](int s) {
+                            const double xe = sh[(12 * s + 6 + cx + 1) * bs + t];
+                            E[s] = pe[s] * xe;                 // (2 beta_a rho_a + rho_dot_a) e_a; not used for the last
+                            return xe;
+                        },
+                        [&](int s) {
+                            const double xs = sh[(12 * s + 9 + cx + 1) * bs + t];
+                            return Limbs58{__double2hiint(xs), __double2loint(xs)};
+                        }, D);
+                    const int e = er + exc - least - 2044 + mc.mix_exp;
                     const bool nan = er == 0x7ff || exc == 0x7ff;      // an infinite or NaN factor
 #pragma unroll
                     for (int s = 0; s < M - 1; ++s) {
