@@ -274,7 +274,8 @@ int lbm_autotune(lbm_ctx *ctx, int trials, int *block_out);
  * lbm_autotune made in an earlier run): blocks[6] in the order of
  * block_out above, each 64, 128 or 256, at most 128 for the moment and
  * species-collision kernels, and 128 for the ghost-node kernel; else
- * LBM_ERR_ARG.  Results do not depend on the choice. */
+ * LBM_ERR_ARG.  Results do not depend on the choice.  (With two or three
+ * species the production-rate entry has no effect, see lbm_step_timed.) */
 int lbm_set_blocks(lbm_ctx *ctx, const int *blocks);
 
 /* lbm_step_async with CUDA events recorded on the stream between the
@@ -284,8 +285,10 @@ int lbm_set_blocks(lbm_ctx *ctx, const int *blocks);
  * gradient, energy-collision and species/mixture-collision kernels over
  * the n steps, phase_ms[LBM_PHASES] the device time from the first launch
  * to the end of the last.  The diffusion velocities, a kernel between the
- * moments and the production rates, are counted with the moments.  Returns
- * like lbm_step. */
+ * moments and the production rates, are counted with the moments; with two
+ * or three species the production rates are part of the energy-collision
+ * kernel and their entry is the time between two events.  Returns like
+ * lbm_step. */
 #define LBM_PHASES 6
 int lbm_step_timed(lbm_ctx *ctx, int n, double *phase_ms);
 

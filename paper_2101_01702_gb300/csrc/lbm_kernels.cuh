@@ -16,7 +16,8 @@
 // cycle): what does not need its range runs in fixed point on the integer pipe
 // or in pairs of floats (lbm_fixed.cuh), to the same accuracy.
 //
-// One time step is six launches on one stream (seven with x ghosts):
+// One time step is six launches on one stream (seven with x ghosts; two fewer
+// with two or three species, see kFewSpecies):
 //   k_ghost  x-face ghost nodes (Sec. 5a; only for non-periodic x)
 //   k_pre    pull, all moments, Newton temperature, relaxation rates, the
 //            local part of the energy-flux correction and the energy
@@ -1599,12 +1600,27 @@ __device__ __forceinline__ void pre_node(const StepArgs &a, const Node &nd, doub
 
 extern __shared__ double sh_pre[];
 
+// With two or three species the step has two launches fewer: the diffusion
+// velocities follow the moments in k_pre, the production rates precede the
+// energy collision in k_step_g.  A kernel's launch and tail, 3 to 4 us, is a
+// twentieth of such a step on a small lattice, and their code is short enough
+// to share a register budget.  Three species, us per step, four kernels / six:
+// 1024 nodes mixed 64.3 / 72.4, fast mixed 59.6 / 68.0, double 94.6 / 99.3
+// (65.0, 61.9 and 152 before the velocities and the rates became kernels of
+// their own); 128^3 mixed 2841 / 2848, fast mixed 2468 / 2501, double 6212 / 6401.
+template <int M>
+constexpr bool kFewSpecies = M < 4;
+
+template <int M, bool FX>
+__device__ __forceinline__ void diff_node(const StepArgs &a, const Node &nd, double *sh, int bs);
+
 template <int M>
 __global__ void __launch_bounds__(LBMK_BLOCK, LBMK_PRE_MINB) k_pre(StepArgs a)
 {
     Node nd;
     if (!node_of(nd, a)) return;
     pre_node<M>(a, nd, sh_pre + threadIdx.x, blockDim.x);
+    if constexpr (kFewSpecies<M>) diff_node<M, false>(a, nd, nullptr, 0);
 }
 
 // ---------------------------------------------------------------------
@@ -1989,6 +2005,7 @@ __global__ void __launch_bounds__(LBMK_MAXBLOCK) k_step_g(StepArgs a)
 {
     Node nd;
     if (!node_of(nd, a)) return;
+    if constexpr (kFewSpecies<M>) chem_node<M>(a, nd.n, sh_chem, blockDim.x);
     collide_energy<M>(a, nd);
 }
 
@@ -2274,6 +2291,7 @@ int launch_one(const StepArgs &a, int k)
         k_pre<M><<<grid_for(a.N, bs), bs, pre_cols<M>() * bs * sizeof(double), a.stream>>>(a);
         constexpr bool FX = kRefined<M, true>;
         static_assert(diff_cols<M, true>() * LBMK_BLOCK * sizeof(double) <= 48 * 1024, "more needs an opt-in");
+        if (kFewSpecies<M>) break;                  // k_pre went on
         if (FX && a.fixed)
             k_diff<M, FX><<<grid_for(a.N, bs), bs, diff_cols<M, FX>() * bs * sizeof(double), a.stream>>>(a);
         else
@@ -2281,6 +2299,7 @@ int launch_one(const StepArgs &a, int k)
         break;
     }
     case LBMK_K_CHEM: {
+        if (kFewSpecies<M>) break;                  // in k_step_g
         static std::atomic<unsigned long long> opted{0};
         const int e = opt_in_smem(k_chem<M>, chem_cols<M>() * LBMK_MAXBLOCK * sizeof(double), opted);
         if (e) return e;
@@ -2288,7 +2307,9 @@ int launch_one(const StepArgs &a, int k)
         break;
     }
     case LBMK_K_GRAD: k_grad<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
-    case LBMK_K_STEPG: k_step_g<M><<<grid_for(a.N, bs), bs, 0, a.stream>>>(a); break;
+    case LBMK_K_STEPG:
+        k_step_g<M><<<grid_for(a.N, bs), bs, kFewSpecies<M> ? chem_cols<M>() * bs * sizeof(double) : 0, a.stream>>>(a);
+        break;
     case LBMK_K_STEP: {
         constexpr bool FX = kFixedStep<M>;
         const int e = FX && a.fixed ? launch_step<M, FX>(a, bs) : launch_step<M, false>(a, bs);
