@@ -70,9 +70,18 @@ enum { LBM_RXN_ELEMENTARY = 0, LBM_RXN_THIRD_BODY = 1, LBM_RXN_FALLOFF = 2 };
  *                   mixture sets as float deviations from per-set rest
  *                   states and collides them in float; their rest
  *                   populations and the energy set stay double, and so do
- *                   the moments, the temperature iteration, the
- *                   Stefan-Maxwell solve, the reaction rates and the
- *                   equilibrium constants;
+ *                   the temperature iteration (its residual; the quotient
+ *                   that scales a correction is a float), the energy
+ *                   equilibria and the equilibrium constants.  The moments
+ *                   of the float populations are float sums of the stored
+ *                   deviations.  What is stored as floats in the end is
+ *                   formed to more than float accuracy: the diffusion
+ *                   velocities from a float elimination refined by a
+ *                   fixed-point residual (2^-40 of the largest n_b |x_b|
+ *                   over the largest n_b; tables outside the fixed-point
+ *                   range and fewer than four species: a double LDL^T
+ *                   solve), the production rates from 58-bit exponents,
+ *                   double rates of progress and sums of 48 bits;
  *   LBM_MIXED_FAST  as LBM_MIXED, but the relaxation rates and the
  *                   Stefan-Maxwell solve run in float, and the exponentials
  *                   of the reported rates (and of a step's, for mechanisms

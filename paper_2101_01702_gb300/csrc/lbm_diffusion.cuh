@@ -1,5 +1,5 @@
-// Stefan-Maxwell diffusion velocities (Eq. (transform1)) without the FP64
-// pipe: a float factorisation and one step of iterative refinement whose
+// Stefan-Maxwell diffusion velocities (Eq. (transform1)) almost without the
+// FP64 pipe: a float factorisation and one step of iterative refinement whose
 // residual is formed in fixed point (lbm_fixed.cuh).  For the mixed unit,
 // where the velocities are stored as floats.
 //
@@ -30,8 +30,8 @@
 // Y_a u cancel).
 //
 // A double LDL^T solve costs 740 FP64 instructions per warp at nine species,
-// 56 thousand cycles of a scheduler; this one about 7 thousand
-// integer and float instructions.
+// 56 thousand cycles of a scheduler; this one about 9 thousand
+// instructions, 36 of them FP64.
 #pragma once
 
 #include "lbm_fixed.cuh"

@@ -7,7 +7,7 @@ Every velocity is finite and the exact one to 2^-24 |x| (rounded to float
 once) plus 2^-40 of the largest n_b |x_b| over the largest n_b (the residual
 sums products n_b x_b in integers, 2^-53 of the largest, and takes its other
 terms as pairs of floats, 2^-46 of each; the float correction adds 2^-22 of
-itself) plus 2^-53 |u| (j - rho u is formed in integers, 2^-56 of the larger)
+itself) plus 2^-53 |u| (j - rho u is one operation in double)
 plus 2^-100 (the floats' range)."""
 import os
 import shutil
