@@ -201,14 +201,14 @@ constexpr int lbmk_block_cand[LBMK_NBLOCKS] = {0, 64, 128, 256};
 
 // The fastest candidate by the times ms (0: not tried), the choice by size
 // where no other is faster by 2 %, more than the timings of a few launches
-// differ; *fixed: the fastest of the others.  Without the choice by size among
+// differ; *fixed: the fastest of the others (64 where no time was measured).  Without the choice by size among
 // the candidates, 48^3 mixed took 452 to 458 us a step tuned and 447 untuned.
 inline int lbmk_choose_block(const float *ms, int *fixed)
 {
     int best = 0;
     for (int j = 1; j < LBMK_NBLOCKS; ++j)
         if (ms[j] > 0.f && (best == 0 || ms[j] < ms[best])) best = j;
-    *fixed = lbmk_block_cand[best];
+    *fixed = lbmk_block_cand[best > 0 ? best : 1];
     return ms[0] > 0.f && (best == 0 || ms[0] <= 1.02f * ms[best]) ? lbmk_block_cand[0] : lbmk_block_cand[best];
 }
 

@@ -28,7 +28,8 @@ def program(tmp_path_factory):
     ((1.0, 1.2, 0.99, 1.3), (0, 128)),      # within what timings differ
     ((1.0, 1.2, 1.1, 0.9), (256, 256)),     # a fixed size is faster
     ((1.0, 0.9, 0.95, 0.0), (64, 64)),      # 256 is not tried for every kernel
-    ((1.0, 1.1, 1.05, 0.0), (0, 128))])
+    ((1.0, 1.1, 1.05, 0.0), (0, 128)),
+    ((0.0, 0.0, 0.0, 0.0), (0, 64))])       # nothing launched (the rates of two or three species)
 def test_choice(program, ms, want):
     r = subprocess.run([str(program), *map(str, ms)], capture_output=True, text=True, check=True)
     assert tuple(int(v) for v in r.stdout.split()) == want
