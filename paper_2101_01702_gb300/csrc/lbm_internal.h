@@ -201,8 +201,9 @@ constexpr int lbmk_block_cand[LBMK_NBLOCKS] = {0, 64, 128, 256};
 
 // The fastest candidate by the times ms (0: not tried), the choice by size
 // where no other is faster by 2 %, more than the timings of a few launches
-// differ; *fixed: the fastest of the others (64 where no time was measured).  Without the choice by size among
-// the candidates, 48^3 mixed took 452 to 458 us a step tuned and 447 untuned.
+// differ; *fixed: the fastest of the others (64 where no time was measured).
+// Without the choice by size among the candidates, 48^3 mixed took 452 to
+// 458 us a step tuned and 447 untuned.
 inline int lbmk_choose_block(const float *ms, int *fixed)
 {
     int best = 0;
